@@ -251,6 +251,12 @@ constexpr int kGradNB = 4;   // neighbour loads in flight per thread (staged gra
 // at 32 % and 61 %, slower at 87 %)
 constexpr double kGradListDensity = 0.75;
 constexpr size_t kGradSmemMax = 160 * 1024;
+// The allowance belongs to the kernel, not to a context: always the largest
+// one, so that a context made later for a mesh of smaller blocks takes nothing
+// from an earlier one.
+cudaError_t allow_smem(const void* kernel) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmemMax);
+}
 
 template <class R> void launch_grad(rt_ctx* ctx) {
   ProfScope ps(ctx, RT_KERNEL_GRAD);
@@ -501,10 +507,8 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
     for (int c0 = 0; c0 < C; c0 += kGradCells) cap = std::max(cap, off[std::min(c0 + kGradCells, C)] - off[c0]);
     const size_t smem = 2 * (size_t)cap * sizeof(float4);
     if (smem <= kGradSmemMax) {
-      CK(cudaFuncSetAttribute(k_grad_staged<kGradNB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-         "staged gradients");
+      CK(allow_smem((const void*)k_grad_staged<kGradNB>), "staged gradients");
       ctx->grad_cap = cap;
-      ctx->grad_smem_attr = (int)smem;
     }
   }
 
@@ -787,14 +791,7 @@ rt_status rt_set_active(rt_ctx* ctx, const uint8_t* active) {
         for (size_t j = j0; j < std::min(j0 + kGradCells, tc.size()); ++j) sum += deg[tc[j]];
         cap_list = std::max(cap_list, sum);
       }
-      const size_t smem = 2 * (size_t)cap_list * sizeof(float4);
-      if (smem > kGradSmemMax) {
-        cap_list = 0;
-      } else if ((int)smem > ctx->grad_smem_attr) {
-        CK(cudaFuncSetAttribute(k_grad_staged<kGradNB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-           "staged gradients");
-        ctx->grad_smem_attr = (int)smem;
-      }
+      if (2 * (size_t)cap_list * sizeof(float4) > kGradSmemMax) cap_list = 0;
     }
     auto up = [&](const void* src, size_t bytes, void** dst) -> rt_status {
       void* p = nullptr;

@@ -58,7 +58,6 @@ struct rt_ctx {
   uint8_t* touched = nullptr;        // per cell: has an active interface
   int n_act = 0, n_touched = 0, n_act_faces = 0, n_grad_blocks = 0;
   int grad_cap_list = 0;             // staged gradients over the touched list: records of the largest block (0: off)
-  int grad_smem_attr = 0;            // dynamic shared memory the staged gradient kernel is allowed
   // work
   void* G = nullptr;           // [C][B][12] in sweep precision
   void* flux = nullptr;        // [F][B] 4-vectors in sweep precision
