@@ -25,39 +25,31 @@ namespace m1rt {
 // transport
 // ---------------------------------------------------------------------------
 
-// Reverse of m1_normal (N D n): lamP -> lamN, lamf (accumulated).  Its
-// quotients by one refined reciprocal per denominator (div_nr).
+// Reverse of N D n = ((s - N) / 3) n + k F, s = sqrt(4 N^2 - 3 |F|^2),
+// k = 3 (F . n) / (2 N + s) (m1_coef): lamP -> lamN, lamf (accumulated).  Two
+// quotients and one square root; smooth at F = 0, where the flux cotangent
+// vanishes by itself.
 __device__ __forceinline__ void m1_normal_vjp(const double v[4], double n0, double n1, double n2, const double lP[3],
                                               double& lN, double lf[3]) {
-  const double fl = sqrt(v[1] * v[1] + v[2] * v[2] + v[3] * v[3]);
   const double lPn = lP[0] * n0 + lP[1] * n1 + lP[2] * n2;
-  if (v[0] > 0.0 && fl > 0.0) {
-    const double iv0 = div_nr(1.0, v[0]), ifl = div_nr(1.0, fl);
-    double f = fl * iv0;
-    const bool clamped = f > 1.0;
-    if (clamped) f = 1.0;
-    const double s = sqrt(4.0 - 3.0 * f * f);
-    const double den = 5.0 + 2.0 * s;
-    const double iden = div_nr(1.0, den);
-    const double chi = (3.0 + 4.0 * f * f) * iden;
-    const double u0 = v[1] * ifl, u1 = v[2] * ifl, u2 = v[3] * ifl;
-    const double un = u0 * n0 + u1 * n1 + u2 * n2;
-    const double a = 0.5 * (1.0 - chi), bb = 0.5 * (3.0 * chi - 1.0);
-    const double lPu = lP[0] * u0 + lP[1] * u1 + lP[2] * u2;
-    lN += a * lPn + bb * un * lPu;
-    const double la = v[0] * lPn, lbb = v[0] * un * lPu;
-    const double lu0 = v[0] * bb * (n0 * lPu + un * lP[0]);
-    const double lu1 = v[0] * bb * (n1 * lPu + un * lP[1]);
-    const double lu2 = v[0] * bb * (n2 * lPu + un * lP[2]);
-    const double lchi = -0.5 * la + 1.5 * lbb;
-    const double dchi = (8.0 * f * den + (3.0 + 4.0 * f * f) * 6.0 * f * div_nr(1.0, s)) * (iden * iden);
-    const double lff = clamped ? 0.0 : lchi * dchi;
-    const double lfl = lff * iv0;
-    lN -= lff * (fl * iv0) * iv0;
-    const double luu = lu0 * u0 + lu1 * u1 + lu2 * u2;
-    lf[0] += (lu0 - luu * u0) * ifl + lfl * u0;
-    lf[1] += (lu1 - luu * u1) * ifl + lfl * u1;
-    lf[2] += (lu2 - luu * u2) * ifl + lfl * u2;
+  const double fl2 = v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
+  if (v[0] > 0.0 && fl2 > 0.0) {
+    const double N2 = v[0] * v[0];
+    double t = fma(-3.0, fl2, 4.0 * N2);
+    t = N2 > t ? N2 : t;
+    const double s = sqrt_nr(t);
+    const double id = div_nr(1.0, fma(2.0, v[0], s)), is = div_nr(1.0, s);
+    const double un = v[1] * n0 + v[2] * n1 + v[3] * n2;
+    const double lPF = lP[0] * v[1] + lP[1] * v[2] + lP[2] * v[3];
+    const double k = 3.0 * un * id;
+    const double ld = -lPF * k * id;                     // of 2 N + s
+    const double third = lPn * (1.0 / 3.0);
+    const double ws = (third + ld) * is;                 // cotangent of s, over s
+    const double lun = 3.0 * lPF * id;
+    lN += 2.0 * ld - third + 4.0 * v[0] * ws;
+    lf[0] += k * lP[0] + lun * n0 - 3.0 * ws * v[1];
+    lf[1] += k * lP[1] + lun * n1 - 3.0 * ws * v[2];
+    lf[2] += k * lP[2] + lun * n2 - 3.0 * ws * v[3];
   } else {
     lN += lPn * (1.0 / 3.0);
   }
@@ -73,13 +65,14 @@ __device__ __forceinline__ void face_pre(const d4& p, const double* __restrict__
   for (int q = 0; q < 4; ++q) v[q] = pc[q] + (Gc[3 * q] * x.x + Gc[3 * q + 1] * x.y + Gc[3 * q + 2] * x.z);
 }
 
-// Clamps of the face state (N >= 0, |F| <= c N), forward.
+// Clamps of the face state (N >= 0, |F| <= c N), forward; the square root
+// only where it clamps.
 __device__ __forceinline__ void face_post(const double pre[4], double v[4]) {
   v[0] = pre[0] < 0.0 ? 0.0 : pre[0];
   v[1] = pre[1]; v[2] = pre[2]; v[3] = pre[3];
-  const double fl = sqrt(v[1] * v[1] + v[2] * v[2] + v[3] * v[3]);
-  if (fl > v[0]) {
-    const double s = fl > 0.0 ? v[0] / fl : 0.0;
+  const double fl2 = v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
+  if (fl2 > v[0] * v[0]) {
+    const double s = v[0] / sqrt(fl2);
     v[1] *= s; v[2] *= s; v[3] *= s;
   }
 }
@@ -88,10 +81,10 @@ __device__ __forceinline__ void face_post(const double pre[4], double v[4]) {
 __device__ __forceinline__ void face_post_vjp(const double pre[4], const double lv[4], double lpre[4]) {
   const bool clampN = pre[0] < 0.0;
   const double v0 = clampN ? 0.0 : pre[0];
-  const double fl = sqrt(pre[1] * pre[1] + pre[2] * pre[2] + pre[3] * pre[3]);
+  const double fl2 = pre[1] * pre[1] + pre[2] * pre[2] + pre[3] * pre[3];
   lpre[0] = lv[0]; lpre[1] = lv[1]; lpre[2] = lv[2]; lpre[3] = lv[3];
-  if (fl > v0) {
-    const double ifl = div_nr(1.0, fl);
+  if (fl2 > v0 * v0) {
+    const double ifl = div_nr(1.0, sqrt(fl2));
     const double lvf = lv[1] * pre[1] + lv[2] * pre[2] + lv[3] * pre[3];
     lpre[0] = lv[0] + lvf * ifl;
 #pragma unroll

@@ -127,20 +127,68 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
-// a / b in FP64 without the FP64 division sequence: an FP32 reciprocal seed
-// (relative error below 2^-22), one Newton-Raphson step y <- y + y (1 - b y)
-// (error ~2^-44), the quotient q = a y and one residual correction
-// q <- q + y (a - b q) (the remainder-based refinement of Markstein, IBM J.
-// Res. Dev. 34 (1990)): within 0.51 units in the last place of a / b, so
-// the correctly rounded quotient but for rare ties.  Five FP64 operations.  Divisors outside the FP32 normal range take the
+// Seed of 1 / x for a normal double x: the FP32 reciprocal of its leading 24
+// bits (in [1, 2)) with the exponent set on the integer pipe, relative error
+// below 2^-22 at any magnitude.  x = 0, subnormal, infinite or NaN, and the
+// extreme exponents whose reciprocal leaves the normal range, return false.
+__device__ __forceinline__ bool rcp_seed(double x, double& y) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int e = (int)((hi >> 20) & 0x7FFu);
+  const float m = __uint_as_float(0x3F800000u | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+  const unsigned r = __float_as_uint(rcp_approx(m));   // in [1/2, 1]
+  const int er = (int)(r >> 23) + 896 - (e - 1023);
+  y = __hiloint2double((int)((hi & 0x80000000u) | ((unsigned)er << 20) | ((r & 0x7FFFFFu) >> 3)), (int)(r << 29));
+  return (unsigned)(e - 64) < 1919u;   // 2^-959 <= |x| < 2^960
+}
+
+// a / b in FP64 without the FP64 division sequence: a reciprocal seed
+// (rcp_seed, relative error below 2^-22), one Newton-Raphson step
+// y <- y + y (1 - b y) (error ~2^-44), the quotient q = a y and one residual
+// correction q <- q + y (a - b q) (the remainder-based refinement of
+// Markstein, IBM J. Res. Dev. 34 (1990)): within 0.51 units in the last
+// place of a / b, so the correctly rounded quotient but for rare ties.  Five
+// FP64 operations at any magnitude of b (photon densities beyond a light
+// front are far below the FP32 range); divisors at the ends of the exponent
+// range, and dividends so small that the remainder would leave it, take the
 // IEEE division.
 __device__ __forceinline__ double div_nr(double a, double b) {
-  const float bf = d2f_int(b);
-  if (!(fabsf(bf) < 1e30f && fabsf(bf) > 1e-30f)) return a / b;
-  double y = f2d_int(rcp_approx(bf));
+  double y;
+  const bool ok = rcp_seed(b, y);
+  const unsigned ha = (unsigned)__double2hiint(a) & 0x7FFFFFFFu;
+  if (!ok || (ha < (64u << 20) && (ha | (unsigned)__double2loint(a)))) return a / b;
   y = fma(y, fma(-b, y, 1.0), y);
   const double q = a * y;
   return fma(y, fma(-b, q, a), q);
+}
+
+// Hardware reciprocal square root approximation (relative error ~2^-22.9).
+__device__ __forceinline__ float rsqrt_approx(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// sqrt(t) in FP64 by Newton's (Heron's) iteration on g -> sqrt(t), each step
+// g <- g + (t - g^2) h with the remainder t - g^2 from one fused multiply-add
+// (Markstein, as div_nr) and h = 1 / (2 sqrt(t)) kept at the seed's 22 bits:
+// the seed's error 2^-22 becomes 2^-43 and then 2^-65, below half a unit in
+// the last place.  Six FP64 operations; the seed is the FP32 reciprocal
+// square root of t's leading 24 bits scaled to [1, 4), its exponent set on
+// the integer pipe.  t = 0, the ends of the exponent range, negative t,
+// infinity and NaN take sqrt().
+__device__ __forceinline__ double sqrt_nr(double t) {
+  const unsigned hi = (unsigned)__double2hiint(t), lo = (unsigned)__double2loint(t);
+  const int e = (int)(hi >> 20);   // sign bit 0 below 2048
+  if (!((unsigned)(e - 128) < 1791u)) return sqrt(t);
+  const int half = (e - 1023) >> 1;             // t = m 4^half, m in [1, 4)
+  const float m = __uint_as_float(((unsigned)(127 + ((e - 1023) & 1)) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+  const unsigned r = __float_as_uint(rsqrt_approx(m));   // in [1/2, 1]
+  const double y = __hiloint2double((int)((((r >> 23) + 896u - (unsigned)half) << 20) | ((r & 0x7FFFFFu) >> 3)),
+                                    (int)(r << 29));
+  double g = t * y;
+  const double h = 0.5 * y;
+  g = fma(fma(-g, g, t), h, g);
+  return fma(fma(-g, g, t), h, g);
 }
 
 // n / d for 0 <= n < 2^31 by one wide multiply and a shift.  With
