@@ -330,12 +330,14 @@ void launch_chem(rt_ctx* ctx, double dt, const ChemTape* tape = nullptr) {
   const int t = 128;
   const int nc = ctx->all_active ? ctx->C : ctx->n_act;
   if (nc == 0) return;
+  // the worklist's persistent grid: room for a group of lanes per cell, two
+  // blocks per SM at most
+  const int nb = (int)std::min<long long>(nblk((long long)nc * kGroup, t), 2 * ctx->n_sm);
   if (!mixed(ctx)) {
     // first attempt of every cell, then the rejected cells (as the mixed path)
     k_chem64_first<<<nblk(nc, t), t, 0, ctx->stream>>>(a, P, ctx->work_cell, ctx->work_f1d, ctx->work_ctl);
     if (!a.do_chem) return;
     ctx->launches++;
-    const int nb = (int)std::min<long long>(nblk(nc, t), ctx->n_sm);
     if (tape)
       k_chem64_rest<true><<<nb, t, 0, ctx->stream>>>(a, P, ctx->work_cell, ctx->work_f1d, ctx->work_ctl, *tape);
     else
@@ -343,14 +345,12 @@ void launch_chem(rt_ctx* ctx, double dt, const ChemTape* tape = nullptr) {
                                                        ChemTape{});
     return;
   }
-  // first attempt of every cell, then the rejected cells (a persistent grid
-  // of one block per SM that takes the worklist 128 entries at a time; the
-  // worklist is short once the gas is near equilibrium)
+  // first attempt of every cell, then the rejected cells (the worklist is
+  // short once the gas is near equilibrium)
   ChemWork w{ctx->work_cell, ctx->work_f1, ctx->work_ctl};
   k_chem_first<<<nblk(nc, t), t, 0, ctx->stream>>>(a, P, ctx->shadow, w);
   if (!a.do_chem) return;
   ctx->launches++;
-  const int nb = (int)std::min<long long>(nblk(nc, t), ctx->n_sm);
   k_chem_rest<<<nb, t, 0, ctx->stream>>>(a, P, ctx->shadow, w);
 }
 

@@ -18,6 +18,7 @@
 // and the chemistry are FP64 in both.
 #pragma once
 #include "rt_chem.cuh"
+#include "rt_chem_coop.cuh"
 
 namespace m1rt {
 
@@ -1133,6 +1134,12 @@ __global__ void k_reciprocal(int n, const double* __restrict__ in, double* out) 
 // carry N and the gas only; the flux is read at the end and scaled by the
 // product of the accepted photon factors.
 
+// A worklist of at most this many cells goes to groups of lanes (rest_groups),
+// a longer one to one thread per cell (rest_threads): a group's attempt has a
+// fraction of the latency but costs the FP64 unit several times as much per
+// cell.
+constexpr int kGroupMax = 4096;
+
 // Worklist of the cells whose first attempt was rejected.
 struct ChemWork {
   int32_t* cell;   // C
@@ -1219,16 +1226,117 @@ __global__ void __launch_bounds__(128, 6) k_chem_first(CellArgs a, ChemParams P,
   w.f1[k] = f1;
 }
 
+// The last warp to finish resets the worklist's counters for the next
+// subcycle.
+__device__ __forceinline__ void rest_done(int* ctl) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) {
+    __threadfence();
+    if (atomicAdd(ctl + 2, 1) == (int)(gridDim.x * (blockDim.x >> 5)) - 1) {
+      ctl[0] = ctl[1] = ctl[2] = 0;
+      __threadfence();
+    }
+  }
+}
+
+// The next entry of the worklist for every group with need: its leader takes
+// one.  The first entries are dealt out so that consecutive ones lie on
+// different SMs.
+__device__ __forceinline__ int group_first() {
+  return (int)((threadIdx.x / kGroup) * gridDim.x + blockIdx.x);
+}
+__device__ __forceinline__ int group_next(int* ctl, bool need, int l) {
+  int k = 0;
+  if (need && l == 0) k = (int)(gridDim.x * (blockDim.x / kGroup)) + atomicAdd(ctl + 1, 1);
+  return from_lane(k, 0);
+}
+
+// A short worklist in the mixed path, one group of lanes per cell (the
+// adaptive loop of chemistry_mixed, resumed after the rejected first attempt;
+// both groups of a warp stay in step, an idle one repeating its last
+// attempt).
+__device__ __forceinline__ void rest_groups(const CellArgs& a, const ChemParams& P, float4* __restrict__ shadow,
+                                            const ChemWork& w, int total) {
+  const int l = threadIdx.x & (kGroup - 1), B = a.B;
+  const size_t C = a.C;
+  const LaneFitF fit = lane_fit_f(l, P.flags);
+  GroupState s{{1.0, 0.0, 1.0, 0.0, 0.0}, 1e4, 0.0, 0.0}, t;
+  GroupCell g;
+  group_cell(P, l, 1.0, g);
+  double rem = 0.0, dt = 0.0;
+  float S = 1.0f;
+  int i = 0, n = 0;
+  const float fmx = (float)P.f_max, fs = (float)P.f_s;
+  auto load = [&](int k) {
+    i = w.cell[k];
+    group_cell(P, l, a.nH[i], g);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) s.x[q] = a.x5[q * C + i];
+    s.T = a.T[i];
+    s.N = l < B ? a.radN[(size_t)i * B + l] : 0.0;
+    rem = a.dt;
+    dt = a.dt * f2d_int(__fdividef(fs, w.f1[k]));
+    S = 1.0f;
+    n = 1;
+  };
+  auto store = [&]() {
+    if (l < B) {
+      const size_t r = (size_t)i * B + l;
+      a.radN[r] = s.N;
+      float4 u = shadow[r];
+      u.x = d2f_int(s.N);
+      u.y *= S; u.z *= S; u.w *= S;
+      shadow[r] = u;
+      if (nonfinite_bits(s.N)) atomicOr(a.status, kStNonFinite);
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+      if (l == q) a.x5[q * C + i] = s.x[q];
+    if (l == 5) a.T[i] = s.T;
+    if (l == 6) a.nsub[i] = n;
+    if (l == 7 && rem > 0) atomicOr(a.status, kStChemSubsteps);
+  };
+  int k = group_first();
+  bool have = k < total;
+  if (have) load(k);
+  for (;;) {
+    const bool done = have && (!positive(rem) || n >= P.max_sub);
+    if (__any_sync(kFull, done)) {
+      if (done) store();
+      k = group_next(w.ctl, done, l);
+      if (done) {
+        have = k < total;
+        if (have) load(k);
+      }
+    } else {
+      if (!__any_sync(kFull, have)) break;
+      double sc;
+      const float f = group_attempt<true>(P, fit, l, g, dt, s, t, sc);
+      if (have) {
+        ++n;
+        if (f > fmx) {
+          dt = dt * (double)__fdividef(fs, f);
+        } else {
+          s = t;
+          S *= d2f_int(sc);
+          rem = __double_as_longlong(dt) == __double_as_longlong(rem) ? 0.0 : rem - dt;
+          dt = dt * (double)(f > 0.0f ? fminf(__fdividef(fs, f), 2.0f) : 2.0f);
+          if (__double_as_longlong(dt) > __double_as_longlong(rem)) dt = rem;
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
 // The worklist's cells, one per thread, handed out 32 at a time to warps.
 // The cells left after the first pass are few and stiff (each runs its own
 // serial chain of attempts, and a warp runs as long as its slowest cell), so
 // the first chunks go to warp 0 of every block -- one warp per SM, each with
 // the SM's FP64 unit to itself -- then to warp 1 of every block, and so on;
 // later chunks go to whichever warp is free.
-__global__ void __launch_bounds__(128) k_chem_rest(CellArgs a, ChemParams P, float4* __restrict__ shadow,
-                                                   ChemWork w) {
-  const int total = *(volatile int*)w.ctl;
-  if (total == 0) return;   // nothing was rejected: the worklist's counters are all zero already
+__device__ __forceinline__ void rest_threads(const CellArgs& a, const ChemParams& P, float4* __restrict__ shadow,
+                                             const ChemWork& w, int total) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int n_warps = gridDim.x * (blockDim.x >> 5);
   // static first chunk: warp-in-block major, so that consecutive chunks lie
@@ -1252,16 +1360,15 @@ __global__ void __launch_bounds__(128) k_chem_rest(CellArgs a, ChemParams P, flo
     if (lane == 0) next = n_warps + atomicAdd(w.ctl + 1, 1);
     chunk = __shfl_sync(0xffffffffu, next, 0);
   }
-  // the last warp to finish resets the worklist for the next subcycle
-  if (lane == 0) {
-    __threadfence();
-    if (atomicAdd(w.ctl + 2, 1) == n_warps - 1) {
-      w.ctl[0] = 0;
-      w.ctl[1] = 0;
-      w.ctl[2] = 0;
-      __threadfence();
-    }
-  }
+}
+
+__global__ void __launch_bounds__(128) k_chem_rest(CellArgs a, ChemParams P, float4* __restrict__ shadow,
+                                                   ChemWork w) {
+  const int total = *(volatile int*)w.ctl;
+  if (total == 0) return;   // nothing was rejected: the worklist's counters are all zero already
+  if (total <= kGroupMax) rest_groups(a, P, shadow, w, total);
+  else rest_threads(a, P, shadow, w, total);
+  rest_done(w.ctl);
 }
 
 // FP64 path: a cell's state (radiation of every bin and gas) in and out.
@@ -1395,15 +1502,135 @@ __global__ void __launch_bounds__(128) k_chem64_first(CellArgs a, ChemParams P, 
   work_f1[k] = f1;
 }
 
-// The FP64 worklist, handed out as k_chem_rest hands out the mixed one.
+// A short worklist in the FP64 path, one group of lanes per cell, as
+// rest_groups.  kTape: also record every attempt, as rest_threads64.
+template <bool kTape>
+__device__ __forceinline__ void rest_groups64(const CellArgs& a, const ChemParams& P,
+                                              const int32_t* __restrict__ work_cell,
+                                              const double* __restrict__ work_f1, int* work_ctl, const ChemTape& tape,
+                                              int total) {
+  const int l = threadIdx.x & (kGroup - 1), B = a.B;
+  const size_t C = a.C;
+  const LaneFit fit = lane_fit(l, P.flags);
+  GroupState s{{1.0, 0.0, 1.0, 0.0, 0.0}, 1e4, 0.0, 0.0}, t;
+  GroupCell g;
+  group_cell(P, l, 1.0, g);
+  double rem = 0.0, dt = 0.0;
+  double* rad = reinterpret_cast<double*>(a.rad);   // (N, f_x, f_y, f_z) per (cell, bin)
+  int i = 0, n = 0;
+  int prev = -1;            // kTape: the cell's last record (the leader's)
+  auto load = [&](int k) {
+    i = work_cell[k];
+    group_cell(P, l, a.nH[i], g);
+#pragma unroll
+    for (int q = 0; q < 5; ++q) s.x[q] = a.x5[q * C + i];
+    s.T = a.T[i];
+    const double* r = rad + (size_t)i * B * 4;
+    s.N = l < B ? r[4 * l] : 0.0;
+    s.f = l < 3 * B ? r[4 * (l / 3) + 1 + l % 3] : 0.0;
+    rem = a.dt;
+    n = 1;
+  };
+  auto store = [&]() {
+    double* r = rad + (size_t)i * B * 4;
+    if (l < B) {
+      r[4 * l] = s.N;
+      if (!isfinite(s.N)) atomicOr(a.status, kStNonFinite);
+    }
+    if (l < 3 * B) r[4 * (l / 3) + 1 + l % 3] = s.f;
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+      if (l == q) a.x5[q * C + i] = s.x[q];
+    if (l == 5) a.T[i] = s.T;
+    if (l == 6) a.nsub[i] = n;
+    if (l == 7 && rem > 0) atomicOr(a.status, kStChemSubsteps);
+    if (kTape && l == 0) tape.last[i] = prev;
+  };
+  // one record of the attempts of each group with rec (past the capacity
+  // nothing is written, the counter still runs): the leader hands it out, the
+  // lanes write the entering state
+  auto begin = [&](bool rec) -> long long {
+    long long cur = 0;
+    if (rec && l == 0) cur = (long long)atomicAdd(tape.used, 1ull);
+    cur = from_lane(cur, 0);
+    if (rec && cur < tape.cap) {
+      ChemRec& r = tape.rec[cur];
+      if (l < B) r.s[l] = s.N;
+      if (l < 3 * B) r.s[B + l] = s.f;
+#pragma unroll
+      for (int q = 0; q < 5; ++q)
+        if (l == q) r.s[4 * B + q] = s.x[q];
+      if (l == 5) r.s[4 * B + 5] = s.T;
+    }
+    return cur;
+  };
+  auto end = [&](long long cur, double len, double f, int flags) {
+    if (l == 0 && cur < tape.cap) {
+      ChemRec& r = tape.rec[cur];
+      r.dt = len; r.f = f; r.cell = i; r.flags = flags; r.prev = prev;
+    }
+    prev = cur < tape.cap ? (int)cur : -1;
+  };
+  // a new cell: its rejected first attempt is recorded too
+  auto take = [&](bool fresh, int k) {
+    if (fresh) load(k);
+    if constexpr (kTape) {
+      const long long cur = begin(fresh);
+      if (fresh) {
+        prev = -1;
+        end(cur, a.dt, work_f1[k], 0);
+      }
+    }
+    if (fresh) dt = a.dt * div_nr(P.f_s, work_f1[k]);
+  };
+  int k = group_first();
+  bool have = k < total;
+  take(have, k);
+  for (;;) {
+    const bool done = have && (!(rem > 0) || n >= P.max_sub);
+    if (__any_sync(kFull, done)) {
+      if (done) store();
+      k = group_next(work_ctl, done, l);
+      if (done) have = k < total;
+      take(done && have, k);
+    } else {
+      if (!__any_sync(kFull, have)) break;
+      long long cur = 0;
+      if constexpr (kTape) cur = begin(have);
+      double sc;
+      const double f = group_attempt<false>(P, fit, l, g, dt, s, t, sc);
+      if (have) {
+        ++n;
+        if (f > P.f_max) {
+          if constexpr (kTape) end(cur, dt, f, 0);
+          dt = dt * div_nr(P.f_s, f);
+        } else {
+          s = t;
+          const double len = dt;
+          rem = (dt == rem) ? 0.0 : rem - dt;
+          double grow = (f > 0) ? div_nr(P.f_s, f) : 2.0;
+          const bool ratio = f > 0 && grow <= 2.0;
+          if (grow > 2.0) grow = 2.0;
+          dt = dt * grow;
+          const bool clipped = dt > rem;
+          if (clipped) dt = rem;
+          if constexpr (kTape)
+            end(cur, len, f, kRecAccepted | (ratio ? kRecRatio : 0) | (clipped ? kRecClipped : 0));
+        }
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// The FP64 worklist, one cell per thread, handed out as rest_threads.
 // kTape: also record every attempt of these cells, the rejected first one
 // included, for the reverse mode.
 template <bool kTape>
-__global__ void __launch_bounds__(128) k_chem64_rest(CellArgs a, ChemParams P, const int32_t* __restrict__ work_cell,
-                                                     const double* __restrict__ work_f1, int* work_ctl,
-                                                     ChemTape tape) {
-  const int total = *(volatile int*)work_ctl;
-  if (total == 0) return;   // nothing was rejected: the worklist's counters are all zero already
+__device__ __forceinline__ void rest_threads64(const CellArgs& a, const ChemParams& P,
+                                               const int32_t* __restrict__ work_cell,
+                                               const double* __restrict__ work_f1, int* work_ctl,
+                                               const ChemTape& tape, int total) {
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int n_warps = gridDim.x * (blockDim.x >> 5);
   int chunk = wib * gridDim.x + blockIdx.x;
@@ -1434,15 +1661,17 @@ __global__ void __launch_bounds__(128) k_chem64_rest(CellArgs a, ChemParams P, c
     if (lane == 0) next = n_warps + atomicAdd(work_ctl + 1, 1);
     chunk = __shfl_sync(0xffffffffu, next, 0);
   }
-  if (lane == 0) {
-    __threadfence();
-    if (atomicAdd(work_ctl + 2, 1) == n_warps - 1) {
-      work_ctl[0] = 0;
-      work_ctl[1] = 0;
-      work_ctl[2] = 0;
-      __threadfence();
-    }
-  }
+}
+
+template <bool kTape>
+__global__ void __launch_bounds__(128) k_chem64_rest(CellArgs a, ChemParams P, const int32_t* __restrict__ work_cell,
+                                                     const double* __restrict__ work_f1, int* work_ctl,
+                                                     ChemTape tape) {
+  const int total = *(volatile int*)work_ctl;
+  if (total == 0) return;   // nothing was rejected: the worklist's counters are all zero already
+  if (total <= kGroupMax) rest_groups64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, total);
+  else rest_threads64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, total);
+  rest_done(work_ctl);
 }
 
 }  // namespace m1rt
