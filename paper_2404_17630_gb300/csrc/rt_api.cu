@@ -155,15 +155,15 @@ rt_status check_config(const rt_config* c) {
 
 template <class R> Geo<R> geo(const rt_ctx* ctx);
 template <> Geo<double> geo<double>(const rt_ctx* c) {
-  return Geo<double>{c->C, c->F, c->B, make_divb(c->B), c->off, c->csr, c->nbr, c->lr, c->nA64, c->rL64, c->rR64, c->w64, c->minv64,
-                     (const d4*)c->hw, (const d4*)c->hx, (const double*)c->xmax, nullptr, nullptr, c->B,
+  return Geo<double>{c->C, c->F, c->B, make_divb(c->B), c->off, c->csr, c->nbr, c->lr, c->nA64, c->rL64, c->rR64,
+                     (const d4*)c->hw, (const d4*)c->hx, c->hx32, (const double*)c->xmax, nullptr, nullptr, c->B,
                      c->touched_cells, c->n_touched,
                      c->grad_blocks, c->n_grad_blocks, c->touched, c->act_faces, c->n_act_faces};
 }
 template <> Geo<float> geo<float>(const rt_ctx* c) {
   // the FP32 sweep reads faces through fa / fb; no per-array face copies
-  return Geo<float>{c->C, c->F, c->B, make_divb(c->B), c->off, c->csr, c->nbr, c->lr, nullptr, nullptr, nullptr, nullptr,
-                    c->minv32, (const float4*)c->hw, (const float4*)c->hx, (const float*)c->xmax, c->fa32, c->fb32,
+  return Geo<float>{c->C, c->F, c->B, make_divb(c->B), c->off, c->csr, c->nbr, c->lr, nullptr, nullptr, nullptr,
+                    (const float4*)c->hw, (const float4*)c->hx, nullptr, (const float*)c->xmax, c->fa32, c->fb32,
                     pad_bins(c->B),
                     c->touched_cells, c->n_touched, c->grad_blocks, c->n_grad_blocks, c->touched, c->act_faces,
                     c->n_act_faces};
@@ -545,12 +545,13 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   }
   AL(ctx->work_cell, C); AL(ctx->work_ctl, 4);
   if (mx) {
-    AL(ctx->fa32, F); AL(ctx->fb32, F); AL(ctx->minv32, 6 * (size_t)C); AL(ctx->ivol, C);
+    AL(ctx->fa32, F); AL(ctx->fb32, F); AL(ctx->ivol, C);
     AL(ctx->work_f1, C);
     AL(ctx->shadow, (size_t)C * B);
     AL(ctx->radN, (size_t)C * B);
   } else {
     AL(ctx->work_f1d, C);
+    AL(ctx->hx32, 2 * (size_t)F);
   }
 #undef AL
   if ((st = copy_in(ctx, ctx->vol, cells->volume, (size_t)C * 8))) return st;
@@ -591,16 +592,17 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
                                                             ctx->fb32);
   }
   if (mx) {
-    k_convert<float><<<nblk(6LL * C), kThreads, 0, ctx->stream>>>(6 * C, ctx->minv64, ctx->minv32);
     k_reciprocal<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->vol, ctx->ivol);
   }
   if (F > 0) {
     if (mx)
       k_build_halfedges<float><<<nblk(2LL * F), kThreads, 0, ctx->stream>>>(
-          2 * F, ctx->csr, ctx->nbr, ctx->w64, ctx->rL64, ctx->rR64, (float4*)ctx->hw, (float4*)ctx->hx);
+          2 * F, ctx->csr, ctx->nbr, ctx->lr, ctx->minv64, ctx->w64, ctx->rL64, ctx->rR64, (float4*)ctx->hw,
+          (float4*)ctx->hx, nullptr);
     else
       k_build_halfedges<double><<<nblk(2LL * F), kThreads, 0, ctx->stream>>>(
-          2 * F, ctx->csr, ctx->nbr, ctx->w64, ctx->rL64, ctx->rR64, (d4*)ctx->hw, (d4*)ctx->hx);
+          2 * F, ctx->csr, ctx->nbr, ctx->lr, ctx->minv64, ctx->w64, ctx->rL64, ctx->rR64, (d4*)ctx->hw, (d4*)ctx->hx,
+          ctx->hx32);
     if (mx)
       k_cell_xmax<float><<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->off, (const float4*)ctx->hx,
                                                                (float*)ctx->xmax);

@@ -27,12 +27,12 @@ struct rt_ctx {
   int2* lr = nullptr;
   d4 *nA64 = nullptr, *rL64 = nullptr, *rR64 = nullptr, *w64 = nullptr;
   void *hw = nullptr, *hx = nullptr;   // half-edge records in the sweep precision
+  float4* hx32 = nullptr;              // FP64 sweep: the half-edges' offsets in FP32
   void* xmax = nullptr;                 // per cell: the largest .w of its offset records (sweep precision)
   double* minv64 = nullptr;
   // FP32 copies (mixed precision)
   f8* fa32 = nullptr;          // FP32 face records (n, A, x_f - s_L, left)
   float4* fb32 = nullptr;      // FP32 face records (x_f - s_R, right)
-  float* minv32 = nullptr;
   // state
   d4* rad = nullptr;      // [C][B] (N, F / c): the FP64 state; mixed precision: the interface records only
   double* radN = nullptr;      // mixed precision: N [C][B] in FP64
