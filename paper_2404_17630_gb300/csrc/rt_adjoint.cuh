@@ -103,10 +103,12 @@ struct AdjArgs {
   const d4* rL;
   const d4* rR;
   const d4* w;
+  const d4* hx;           // half-edges: face-centre offsets of their cell
   const double* minv;
-  const double* vol;
+  const double* ivol;     // 1 / V
   const d4* rad;          // state before the transport pass
   const double* G;        // its limited gradients
+  const GradTape* tape;   // and what k_grad recorded beside them
   const d4* lam_out;      // cotangent of the state after the pass
   d4* lampre;             // [F][B][2] cotangents of the extrapolated face states
   d4* lamr;               // [C][B][3] cotangents of the least-squares right-hand sides
@@ -115,8 +117,7 @@ struct AdjArgs {
   d4* lam_part;           // [C][B] partial cotangent of the state before the pass
   d4* lam_in;             // [C][B] result: cotangent of the state before the pass
   double lam;             // c_red dt / unit_length_cm
-  int order, limiter;
-  double lim_eps2;
+  int order;
 };
 
 __global__ void __launch_bounds__(256) k_adj_face(AdjArgs a) {
@@ -128,9 +129,9 @@ __global__ void __launch_bounds__(256) k_adj_face(AdjArgs a) {
   const d4 nA = a.nA[f];
   const size_t sL = (size_t)c.x * B + b, sR = (size_t)c.y * B + b;
   const d4 lo_L = a.lam_out[sL], lo_R = a.lam_out[sR];
-  const double iVL = div_nr(1.0, a.vol[c.x]), iVR = div_nr(1.0, a.vol[c.y]);
-  double lout[4] = {a.lam * (lo_R.x * iVR - lo_L.x * iVL), a.lam * (lo_R.y * iVR - lo_L.y * iVL),
-                    a.lam * (lo_R.z * iVR - lo_L.z * iVL), a.lam * (lo_R.w * iVR - lo_L.w * iVL)};
+  const double iVL = a.lam * a.ivol[c.x], iVR = a.lam * a.ivol[c.y];
+  double lout[4] = {lo_R.x * iVR - lo_L.x * iVL, lo_R.y * iVR - lo_L.y * iVL, lo_R.z * iVR - lo_L.z * iVL,
+                    lo_R.w * iVR - lo_L.w * iVL};
   double preL[4], preR[4], vL[4], vR[4];
   face_pre(a.rad[sL], a.G + sL * 12, a.rL[f], preL);
   face_pre(a.rad[sR], a.G + sR * 12, a.rR[f], preR);
@@ -157,8 +158,10 @@ __global__ void __launch_bounds__(256) k_adj_face(AdjArgs a) {
   a.lampre[(size_t)t * 2 + 1] = make_d4(pR[0], pR[1], pR[2], pR[3]);
 }
 
-__device__ __forceinline__ double d4c(const d4& v, int q) { return q == 0 ? v.x : (q == 1 ? v.y : (q == 2 ? v.z : v.w)); }
-
+// The gradients before the limiter, its factors and the limiting faces come
+// from k_grad's record of the same state (192 bytes read instead of the
+// least-squares sums and a quotient per face and component formed again, which
+// were two thirds of this kernel's FP64 instructions).
 __global__ void __launch_bounds__(256) k_adj_cellgrad(AdjArgs a) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int B = a.B;
@@ -168,10 +171,11 @@ __global__ void __launch_bounds__(256) k_adj_cellgrad(AdjArgs a) {
   const d4 lo = a.lam_out[t];
   double lU[4] = {lo.x, lo.y, lo.z, lo.w};
   double lG[4][3] = {};
+#pragma unroll 2
   for (int k = k0; k < k1; ++k) {
-    const int e = a.csr[k], f = e >> 1, side = e & 1;
-    const d4 lp = a.lampre[((size_t)f * B + b) * 2 + side];
-    const d4 x = side ? a.rR[f] : a.rL[f];
+    const int e = a.csr[k];
+    const d4 lp = a.lampre[((size_t)(e >> 1) * B + b) * 2 + (e & 1)];
+    const d4 x = a.hx[k];
     const double l4[4] = {lp.x, lp.y, lp.z, lp.w};
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -185,61 +189,26 @@ __global__ void __launch_bounds__(256) k_adj_cellgrad(AdjArgs a) {
   double coef[4] = {0, 0, 0, 0};
   int jst[4] = {-1, -1, -1, -1};
   if (a.order >= 2) {
-    const d4 pi4 = a.rad[t];
-    double r[4][3] = {}, mx[4], mn[4];
-    int jmx[4], jmn[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) { mx[q] = mn[q] = d4c(pi4, q); jmx[q] = jmn[q] = i; }
-    for (int k = k0; k < k1; ++k) {
-      const int e = a.csr[k], f = e >> 1;
-      const int j = a.nbr[k];
-      const d4 pj = a.rad[(size_t)j * B + b];
-      const d4 w = a.w[f];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double vj = d4c(pj, q), vi = d4c(pi4, q);
-        const double dphi = (e & 1) ? (vi - vj) : (vj - vi);
-        r[q][0] += w.x * dphi; r[q][1] += w.y * dphi; r[q][2] += w.z * dphi;
-        if (vj > mx[q]) { mx[q] = vj; jmx[q] = j; }
-        if (vj < mn[q]) { mn[q] = vj; jmn[q] = j; }
-      }
-    }
+    const GradTape& r = a.tape[t];
     const double* m = a.minv + 6 * (size_t)i;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      double g[3];
-      g[0] = m[0] * r[q][0] + m[1] * r[q][1] + m[2] * r[q][2];
-      g[1] = m[1] * r[q][0] + m[3] * r[q][1] + m[4] * r[q][2];
-      g[2] = m[2] * r[q][0] + m[4] * r[q][1] + m[5] * r[q][2];
       double lg[3] = {lG[q][0], lG[q][1], lG[q][2]};
-      if (a.limiter) {
-        const double vi = d4c(pi4, q);
-        const double gg = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
-        double psi = 1.0, dstar = 0.0, xs[3] = {0, 0, 0};
-        int js = -1;
-        for (int k = k0; k < k1; ++k) {
-          const int e = a.csr[k], f = e >> 1;
-          const d4 x = (e & 1) ? a.rR[f] : a.rL[f];
-          const double dphi = g[0] * x.x + g[1] * x.y + g[2] * x.z;
-          const double xx = x.x * x.x + x.y * x.y + x.z * x.z;
-          if (dphi * dphi > a.lim_eps2 * gg * xx) {
-            const double lim = div_nr(dphi > 0.0 ? mx[q] - vi : mn[q] - vi, dphi);
-            if (lim < psi) {
-              psi = lim; dstar = dphi; xs[0] = x.x; xs[1] = x.y; xs[2] = x.z;
-              js = dphi > 0.0 ? jmx[q] : jmn[q];
-            }
-          }
-        }
-        if (js >= 0) {
-          const double sdot = lG[q][0] * g[0] + lG[q][1] * g[1] + lG[q][2] * g[2];
-          const double sd = div_nr(sdot, dstar);
-#pragma unroll
-          for (int d = 0; d < 3; ++d) lg[d] = psi * lG[q][d] - sd * psi * xs[d];
-          if (js != i) {
-            lU[q] -= sd;
-            coef[q] = sd;
-            jst[q] = js;
-          }
+      const int at = r.at[q];
+      if (at >= 0) {
+        // psi = (extreme - value) / (g . x) on the limiting face
+        const double g0 = r.g[3 * q], g1 = r.g[3 * q + 1], g2 = r.g[3 * q + 2], psi = r.psi[q];
+        const d4 x = a.hx[at];
+        const double dstar = g0 * x.x + g1 * x.y + g2 * x.z;
+        const double sd = div_nr(lG[q][0] * g0 + lG[q][1] * g1 + lG[q][2] * g2, dstar);
+        const double sp = sd * psi;
+        lg[0] = psi * lG[q][0] - sp * x.x;
+        lg[1] = psi * lG[q][1] - sp * x.y;
+        lg[2] = psi * lG[q][2] - sp * x.z;
+        if (r.cell[q] != i) {
+          lU[q] -= sd;
+          coef[q] = sd;
+          jst[q] = r.cell[q];
         }
       }
       lr_out[q][0] = m[0] * lg[0] + m[1] * lg[1] + m[2] * lg[2];
@@ -251,11 +220,8 @@ __global__ void __launch_bounds__(256) k_adj_cellgrad(AdjArgs a) {
   lr4[0] = make_d4(lr_out[0][0], lr_out[0][1], lr_out[0][2], lr_out[1][0]);
   lr4[1] = make_d4(lr_out[1][1], lr_out[1][2], lr_out[2][0], lr_out[2][1]);
   lr4[2] = make_d4(lr_out[2][2], lr_out[3][0], lr_out[3][1], lr_out[3][2]);
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    a.lim_coef[(size_t)t * 4 + q] = coef[q];
-    a.lim_cell[(size_t)t * 4 + q] = jst[q];
-  }
+  reinterpret_cast<d4*>(a.lim_coef)[t] = make_d4(coef[0], coef[1], coef[2], coef[3]);
+  reinterpret_cast<int4*>(a.lim_cell)[t] = make_int4(jst[0], jst[1], jst[2], jst[3]);
   a.lam_part[t] = make_d4(lU[0], lU[1], lU[2], lU[3]);
 }
 
@@ -265,6 +231,10 @@ __device__ __forceinline__ void load_lamr(const d4* lamr, size_t t, double o[12]
   o[6] = b.z; o[7] = b.w; o[8] = c.x; o[9] = c.y; o[10] = c.z; o[11] = c.w;
 }
 
+// The right-hand side's term w (phi_j - phi_i) of a face enters the sums of
+// both its cells with the same sign of w: cell i's share is -+ w . (lamr_i +
+// lamr_j), and its own part, lamr_i . sum -+ w, needs the sum of the weights
+// only.
 __global__ void __launch_bounds__(256) k_adj_cellsum(AdjArgs a) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int B = a.B;
@@ -273,23 +243,31 @@ __global__ void __launch_bounds__(256) k_adj_cellsum(AdjArgs a) {
   const d4 p = a.lam_part[t];
   double lU[4] = {p.x, p.y, p.z, p.w};
   if (a.order >= 2) {
-    for (int k = a.off[i]; k < a.off[i + 1]; ++k) {
-      const int e = a.csr[k], f = e >> 1;
-      const int j = a.nbr[k];
-      const int2 c = a.lr[f];
-      double rl[12], rr[12];
-      load_lamr(a.lamr, (size_t)c.x * B + b, rl);
-      load_lamr(a.lamr, (size_t)c.y * B + b, rr);
-      const d4 w = a.w[f];
+    double W[3] = {0.0, 0.0, 0.0}, o[12];
+    const int k0 = a.off[i], k1 = a.off[i + 1];
+#pragma unroll 2
+    for (int k = k0; k < k1; ++k) {
+      const int e = a.csr[k];
+      const size_t jb = (size_t)a.nbr[k] * B + b;
+      const d4 w = a.w[e >> 1];
+      load_lamr(a.lamr, jb, o);
+      const int4 lc = reinterpret_cast<const int4*>(a.lim_cell)[jb];
       const double sg = (e & 1) ? 1.0 : -1.0;
+      const double wx = sg * w.x, wy = sg * w.y, wz = sg * w.z;
+      W[0] += wx; W[1] += wy; W[2] += wz;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        lU[q] += sg * (w.x * (rl[3 * q] + rr[3 * q]) + w.y * (rl[3 * q + 1] + rr[3 * q + 1]) +
-                       w.z * (rl[3 * q + 2] + rr[3 * q + 2]));
-        const size_t jq = ((size_t)j * B + b) * 4 + q;
-        if (a.lim_cell[jq] == i) lU[q] += a.lim_coef[jq];
+      for (int q = 0; q < 4; ++q) lU[q] += wx * o[3 * q] + wy * o[3 * q + 1] + wz * o[3 * q + 2];
+      if (lc.x == i || lc.y == i || lc.z == i || lc.w == i) {
+        const d4 c = reinterpret_cast<const d4*>(a.lim_coef)[jb];
+        if (lc.x == i) lU[0] += c.x;
+        if (lc.y == i) lU[1] += c.y;
+        if (lc.z == i) lU[2] += c.z;
+        if (lc.w == i) lU[3] += c.w;
       }
     }
+    load_lamr(a.lamr, t, o);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) lU[q] += W[0] * o[3 * q] + W[1] * o[3 * q + 1] + W[2] * o[3 * q + 2];
   }
   a.lam_in[t] = make_d4(lU[0], lU[1], lU[2], lU[3]);
 }

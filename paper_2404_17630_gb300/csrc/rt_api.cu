@@ -283,7 +283,7 @@ template <class R> void launch_grad(rt_ctx* ctx) {
   const long long n = (long long)(ctx->all_active ? ctx->C : ctx->n_touched) * ctx->B;
   if (n == 0) return;
   k_grad<R><<<nblk(n), kThreads, 0, ctx->stream>>>(geo<R>(ctx), sweep_rad<R>(ctx), (R*)ctx->G, ctx->cfg.order,
-                                                   ctx->cfg.limiter, e * e);
+                                                   ctx->cfg.limiter, e * e, nullptr);
 }
 
 template <class R> void launch_flux(rt_ctx* ctx) {
@@ -543,9 +543,9 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
     if (e != cudaSuccess) return cuda_fail(ctx, e, "half-edges");
     ctx->allocs.push_back(p); ctx->xmax = p;
   }
-  AL(ctx->work_cell, C); AL(ctx->work_ctl, 4);
+  AL(ctx->work_cell, C); AL(ctx->work_ctl, 4); AL(ctx->ivol, C);
   if (mx) {
-    AL(ctx->fa32, F); AL(ctx->fb32, F); AL(ctx->ivol, C);
+    AL(ctx->fa32, F); AL(ctx->fb32, F);
     AL(ctx->work_f1, C);
     AL(ctx->shadow, (size_t)C * B);
     AL(ctx->radN, (size_t)C * B);
@@ -591,9 +591,7 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
     k_build_facerecs<<<nblk(F), kThreads, 0, ctx->stream>>>(F, ctx->lr, ctx->nA64, ctx->rL64, ctx->rR64, ctx->fa32,
                                                             ctx->fb32);
   }
-  if (mx) {
-    k_reciprocal<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->vol, ctx->ivol);
-  }
+  k_reciprocal<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->vol, ctx->ivol);
   if (F > 0) {
     if (mx)
       k_build_halfedges<float><<<nblk(2LL * F), kThreads, 0, ctx->stream>>>(
@@ -1165,6 +1163,9 @@ rt_status adj_prepare(rt_ctx* ctx, int nseg, int k) {
   AA(A.lam_x5, 5 * C); AA(A.lam_T, C); AA(A.lam_nH, C); AA(A.lam_S, B * C); AA(A.lim_coef, C * B * 4);
   AA(A.lim_cell, C * B * 4);
   AA(A.tape_last, (size_t)k * C); AA(A.tape_used, 1);
+  GradTape* gt = nullptr;
+  AA(gt, C * B);
+  A.grad = gt;
 #undef AA
   const long long first = std::max<long long>(4096, (long long)C / 4);
   if ((st = tape_grow(ctx, first, first, 0))) return st;
@@ -1191,12 +1192,14 @@ rt_status adj_copy_state(rt_ctx* ctx, d4* rad, double* x5, double* T, bool save)
 AdjArgs adj_args(rt_ctx* ctx, const d4* rad, double dt) {
   AdjArgs a;
   a.C = ctx->C; a.F = ctx->F; a.B = ctx->B; a.off = ctx->off; a.csr = ctx->csr; a.nbr = ctx->nbr; a.lr = ctx->lr;
-  a.nA = ctx->nA64; a.rL = ctx->rL64; a.rR = ctx->rR64; a.w = ctx->w64; a.minv = ctx->minv64; a.vol = ctx->vol;
+  a.nA = ctx->nA64; a.rL = ctx->rL64; a.rR = ctx->rR64; a.w = ctx->w64;
+  a.hx = (const d4*)ctx->hx; a.minv = ctx->minv64; a.ivol = ctx->ivol;
+  a.tape = (const GradTape*)ctx->adj.grad;
   a.rad = rad; a.G = (const double*)ctx->G; a.lam_out = ctx->adj.lam_rad; a.lampre = ctx->adj.lampre;
   a.lamr = ctx->adj.lamr; a.lim_coef = ctx->adj.lim_coef; a.lim_cell = ctx->adj.lim_cell;
   a.lam_part = ctx->adj.lam_part; a.lam_in = ctx->adj.lam_in;
   a.lam = ctx->cfg.c_red * dt / ctx->cfg.unit_length_cm;
-  a.order = ctx->cfg.order; a.limiter = ctx->cfg.limiter; a.lim_eps2 = ctx->cfg.lim_eps * ctx->cfg.lim_eps;
+  a.order = ctx->cfg.order;
   return a;
 }
 
@@ -1223,9 +1226,9 @@ rt_status adj_subcycle(rt_ctx* ctx, int slot, double dts) {
   const long long nCB = (long long)C * B, nFB = (long long)ctx->F * B;
   const d4* rt_rad = A.tp_rad_trans + slot * C * B;
   // gradients of the recorded state
-  k_grad<double><<<nblk(nCB), kThreads, 0, ctx->stream>>>(
+  k_grad<double, true><<<nblk(nCB), kThreads, 0, ctx->stream>>>(
       geo<double>(ctx), rt_rad, (double*)ctx->G, ctx->cfg.order, ctx->cfg.limiter,
-      ctx->cfg.lim_eps * ctx->cfg.lim_eps);
+      ctx->cfg.lim_eps * ctx->cfg.lim_eps, (GradTape*)A.grad);
   AdjArgs a = adj_args(ctx, rt_rad, dts);
   k_adj_face<<<nblk(nFB), kThreads, 0, ctx->stream>>>(a);
   k_adj_cellgrad<<<nblk(nCB), kThreads, 0, ctx->stream>>>(a);

@@ -110,6 +110,7 @@ struct rt_ctx {
     d4 *ck_rad = nullptr, *tp_rad_chem = nullptr, *tp_rad_trans = nullptr, *fin_rad = nullptr;
     double *ck_x5 = nullptr, *ck_T = nullptr, *tp_x5 = nullptr, *tp_T = nullptr, *fin_x5 = nullptr, *fin_T = nullptr;
     d4 *lam_rad = nullptr, *lam_part = nullptr, *lam_in = nullptr, *lampre = nullptr, *lamr = nullptr;
+    void* grad = nullptr;                      // GradTape of every (cell, bin)
     double *lam_x5 = nullptr, *lam_T = nullptr, *lam_nH = nullptr, *lam_S = nullptr, *lim_coef = nullptr;
     int32_t* lim_cell = nullptr;
     int32_t* tape_last = nullptr;              // [k][C] last chemistry record of each cell, per subcycle

@@ -325,12 +325,11 @@ __device__ __forceinline__ bool scaled_f32(const double g[3], float o[3]) {
 // folded into the weights: 0.85 -> 0.54 ms per launch at 250,047 cells).  Where a lead is
 // smaller (faces that tie by symmetry; a leader within the band of zero) every
 // face's product is formed in FP64.  A component without gradient has no
-// extremes.
+// extremes.  at[2q], at[2q + 1]: the first face that attains dpos[q], dneg[q].
 __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const float4* __restrict__ xf, int k0, int k1,
                                              const double gr[4][3], const double thr[4], double X, double dpos[4],
-                                             double dneg[4]) {
+                                             double dneg[4], int at[8]) {
   float gf[4][3], m1[8], m2[8];
-  int at[8];
   bool flat[4], sure = true;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -379,8 +378,11 @@ __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const fl
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const double dphi = gr[q][0] * x.x + gr[q][1] * x.y + gr[q][2] * x.z;
-        bpos[q] = max_bits_pos(bpos[q], dphi);
-        bneg[q] = max_bits_neg(bneg[q], dphi);
+        const long long p = max_bits_pos(bpos[q], dphi), n = max_bits_neg(bneg[q], dphi);
+        at[2 * q] = p != bpos[q] ? k : at[2 * q];
+        at[2 * q + 1] = n != bneg[q] ? k : at[2 * q + 1];
+        bpos[q] = p;
+        bneg[q] = n;
       }
     }
   }
@@ -402,8 +404,11 @@ __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const fl
       for (int q = 0; q < 4; ++q) {
         const double dphi = gr[q][0] * x.x + gr[q][1] * x.y + gr[q][2] * x.z;
         if (__double_as_longlong(dphi * dphi) > __double_as_longlong(thr[q] * x.w)) {
-          bpos[q] = max_bits_pos(bpos[q], dphi);
-          bneg[q] = max_bits_neg(bneg[q], dphi);
+          const long long p = max_bits_pos(bpos[q], dphi), n = max_bits_neg(bneg[q], dphi);
+          at[2 * q] = p != bpos[q] ? k : at[2 * q];
+          at[2 * q + 1] = n != bneg[q] ? k : at[2 * q + 1];
+          bpos[q] = p;
+          bneg[q] = n;
         }
       }
     }
@@ -426,10 +431,20 @@ template <class R> __device__ __forceinline__ R rmin(R a, R b) {
   else return b < a ? b : a;
 }
 
+// What the reverse mode needs of a (cell, bin)'s gradients beside the limited
+// ones: the gradients before the limiter, the factors, the half-edge that
+// limits each component (-1: none) and the cell that holds the extreme it is
+// limited by.
+struct GradTape {
+  double g[12], psi[4];
+  int32_t at[4], cell[4];
+};
+
 // G[(i*B + b)*12 + q*3 + d]: limited gradient of component q of bin b.
-template <class R>
+// kTape (FP64 sweep): the reverse mode's record too.
+template <class R, bool kTape = false>
 __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict__ rad, R* __restrict__ G,
-                                              int order, int limiter, R lim_eps2) {
+                                              int order, int limiter, R lim_eps2, GradTape* __restrict__ tape) {
   int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int B = g.B;
   if (t >= (g.clist ? g.nc : g.C) * B) return;
@@ -447,7 +462,7 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
 #pragma unroll
       for (int k = 0; k < 12; ++k) Go[k] = R(0);
     }
-    return;
+    return;   // first order: the reverse mode reads no record either
   }
   R gr[4][3];
   R mx[4], mn[4];
@@ -457,11 +472,13 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
   // is what bounds this kernel).  Rounding is monotone, so max_j fl(phi_j -
   // phi_i) = fl(max_j phi_j - phi_i): the same values as the definition.
   long long dmx[4], dmn[4];   // bits of the largest difference, magnitude bits of the most negative
+  int jmx[4], jmn[4];         // kTape: the cells they belong to
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     gr[q][0] = gr[q][1] = gr[q][2] = R(0);
     mx[q] = mn[q] = comp<R>(pi, q);
     dmx[q] = dmn[q] = 0;
+    jmx[q] = jmn[q] = i;
   }
   const int k0 = g.off[i], k1 = g.off[i + 1];
   // half-edge k: u_k (phi_j - phi_i) is this face's term of the gradient
@@ -473,8 +490,13 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
       gr[q][1] += hw.y * dphi;
       gr[q][2] += hw.z * dphi;
       if constexpr (sizeof(R) == 8) {
-        dmx[q] = max_bits_pos(dmx[q], dphi);
-        dmn[q] = max_bits_neg(dmn[q], dphi);
+        const long long up = max_bits_pos(dmx[q], dphi), dn = max_bits_neg(dmn[q], dphi);
+        if constexpr (kTape) {
+          jmx[q] = up != dmx[q] ? bits_id(hw.w) : jmx[q];
+          jmn[q] = dn != dmn[q] ? bits_id(hw.w) : jmn[q];
+        }
+        dmx[q] = up;
+        dmn[q] = dn;
       } else {
         mx[q] = rmax<R>(mx[q], vj);
         mn[q] = rmin<R>(mn[q], vj);
@@ -490,6 +512,7 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
     acc_face(hw, ld4<R>(rad + (size_t)bits_id(hw.w) * B + b));
   }
   R gg[4], psi[4];
+  int lim_at[4] = {-1, -1, -1, -1}, lim_cell[4] = {-1, -1, -1, -1};
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     gg[q] = gr[q][0] * gr[q][0] + gr[q][1] * gr[q][1] + gr[q][2] * gr[q][2];
@@ -502,6 +525,7 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
     // (most negative) g.x: two divisions per component instead of one per
     // face, with bitwise the same result.
     R dpos[4], dneg[4];
+    int at[8];
     if constexpr (sizeof(R) == 4) {
       float eg[4];
 #pragma unroll
@@ -511,7 +535,7 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
       R thr[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) thr[q] = lim_eps2 * gg[q];
-      lim_extremes(g.hx, g.hx32, k0, k1, gr, thr, __ldg(g.xmax + i), dpos, dneg);
+      lim_extremes(g.hx, g.hx32, k0, k1, gr, thr, __ldg(g.xmax + i), dpos, dneg, at);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -529,10 +553,17 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
         // tests on the integer pipe
         if (gt_nonneg(dpos[q], 0.0)) {
           const R lim = div_nr(up, dpos[q]);
+          if (kTape && gt_nonneg(psi[q], lim)) { lim_at[q] = at[2 * q]; lim_cell[q] = jmx[q]; }
           psi[q] = gt_nonneg(psi[q], lim) ? lim : psi[q];
         }
         if (__double_as_longlong(dneg[q]) != 0) {
           const R lim = div_nr(dn, dneg[q]);
+          // equal factors: the face that comes first
+          if (kTape && (gt_nonneg(psi[q], lim) ||
+                        (lim_at[q] > at[2 * q + 1] && __double_as_longlong(psi[q]) == __double_as_longlong(lim)))) {
+            lim_at[q] = at[2 * q + 1];
+            lim_cell[q] = jmn[q];
+          }
           psi[q] = gt_nonneg(psi[q], lim) ? lim : psi[q];
         }
       } else {
@@ -546,6 +577,16 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
         }
       }
     }
+  }
+  if constexpr (kTape) {
+    GradTape& r = tape[t];
+    d4* r4 = reinterpret_cast<d4*>(&r);
+    r4[0] = make_d4(gr[0][0], gr[0][1], gr[0][2], gr[1][0]);
+    r4[1] = make_d4(gr[1][1], gr[1][2], gr[2][0], gr[2][1]);
+    r4[2] = make_d4(gr[2][2], gr[3][0], gr[3][1], gr[3][2]);
+    r4[3] = make_d4(psi[0], psi[1], psi[2], psi[3]);
+    reinterpret_cast<int4*>(r.at)[0] = make_int4(lim_at[0], lim_at[1], lim_at[2], lim_at[3]);
+    reinterpret_cast<int4*>(r.cell)[0] = make_int4(lim_cell[0], lim_cell[1], lim_cell[2], lim_cell[3]);
   }
   R o[12];
 #pragma unroll
