@@ -282,19 +282,13 @@ const char *rt_fp64_peak_last_error(void);
  * memory); anything else, device memory of another GPU included, gets
  * RT_INVALID_ARG before anything is enqueued.  The arrays must describe a
  * valid mesh (ids in range); they are not checked.
- * Its only scratch is a static device array of 6 doubles per cell for at
- * most 262144 cells (12.6 MB held on every GPU that loads the library until
- * the process exits); larger meshes get RT_INVALID_ARG.  Nothing is
- * allocated.  The first call on a device looks up that array's device
- * address (cudaGetSymbolAddress) and caches it with the device's current
- * context; a call made after that context was replaced (cudaDeviceReset)
- * looks it up again.  Make the first call on a device, and the first after
- * a reset, before any stream capture.  All calls on a device share the
- * array: work enqueued by calls that may overlap on the GPU (other streams,
- * unordered host threads) races.  Asynchronous on stream; host-side errors
- * and failed launches of its own kernels are returned as status codes, with
- * a message from rt_noalloc_last_error(); an error the caller left pending
- * in the CUDA runtime is neither reported nor cleared. */
+ * At most 262144 cells; larger meshes get RT_INVALID_ARG.  Nothing is
+ * allocated and no device memory outside the caller's arrays is used, so
+ * calls with different outputs may overlap.  Asynchronous on stream;
+ * host-side errors and failed launches of its own kernels are returned as
+ * status codes, with a message from rt_noalloc_last_error(); an error the
+ * caller left pending in the CUDA runtime is neither reported nor cleared.
+ */
 rt_status rt_gradients_noalloc(const rt_cells *cells, const rt_faces *faces, const int32_t *cell_off,
                                const int32_t *cell_faces, int n_bins, int order, int limiter, double lim_eps,
                                double box, const double *N, const double *F_red, double *G, int *bad_cell,

@@ -19,6 +19,7 @@
 #pragma once
 #include "rt_chem.cuh"
 #include "rt_chem_coop.cuh"
+#include "rt_limiter.cuh"
 
 namespace m1rt {
 
@@ -220,35 +221,6 @@ template <class R> __device__ __forceinline__ R comp(const R4<R>& v, int q) {
   return q == 0 ? v.x : (q == 1 ? v.y : (q == 2 ? v.z : v.w));
 }
 
-// Running extremes of FP64 differences on the integer pipe.  The bits of a
-// double x >= +0 order like x as signed 64-bit integers and those of x < 0
-// are negative, so max(bits, bits(d)) keeps the largest d >= 0 (start: +0);
-// the magnitude bits of d < 0 (0 for d >= 0) track the most negative d.
-__device__ __forceinline__ long long max_bits_pos(long long b, double d) {
-  const long long v = __double_as_longlong(d);
-  return v > b ? v : b;
-}
-__device__ __forceinline__ long long max_bits_neg(long long m, double d) {
-  const long long v = __double_as_longlong(d);
-  const long long mag = (v & 0x7FFFFFFFFFFFFFFFLL) & (v >> 63);
-  return mag > m ? mag : m;
-}
-// -magnitude from max_bits_neg, +0 where nothing was negative
-__device__ __forceinline__ double neg_from_bits(long long m) {
-  return __longlong_as_double(m ? (m | (long long)0x8000000000000000ULL) : 0LL);
-}
-
-// FP64 comparisons on the integer pipe, exact for the values they are used
-// on: a > b for a, b >= +0 (the bit patterns order like the values), and
-// x < 0 (negative, not -0, not NaN).
-__device__ __forceinline__ bool gt_nonneg(double a, double b) {
-  return __double_as_longlong(a) > __double_as_longlong(b);
-}
-__device__ __forceinline__ bool lt_zero(double x) {
-  const long long b = __double_as_longlong(x), m = b & 0x7FFFFFFFFFFFFFFFLL;
-  return b < 0 && m != 0 && m <= 0x7FF0000000000000LL;
-}
-
 // Limiter extremes of one (cell, bin) over its faces k0..k1-1: dpos =
 // max(0, max g.x_f) and dneg = min(0, min g.x_f) over the faces that pass
 // the regularisation test |g.x_f| > eps |g| |x_f|.  First one pass without
@@ -289,134 +261,6 @@ __device__ __forceinline__ void lim_extremes(const float4* __restrict__ xs, int 
       dpos[q] = fmaxf(dpos[q], dm);
       dneg[q] = fminf(dneg[q], dm);
     }
-  }
-}
-
-// g scaled by a power of two so that its largest component lies in [1, 2),
-// cut to FP32 on the integer pipe (relative error below 2^-23; components
-// 2^-126 of the largest become zero).  false where that has no meaning: g = 0,
-// subnormal or not finite.
-__device__ __forceinline__ bool scaled_f32(const double g[3], float o[3]) {
-  unsigned hi[3], top = 0;
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    hi[d] = (unsigned)__double2hiint(g[d]);
-    const unsigned e = hi[d] & 0x7FF00000u;
-    top = e > top ? e : top;
-  }
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    const int e = (int)((hi[d] & 0x7FF00000u) >> 20) - (int)(top >> 20) + 127;
-    const unsigned m = ((hi[d] & 0xFFFFFu) << 3) | ((unsigned)__double2loint(g[d]) >> 29);
-    o[d] = __uint_as_float((hi[d] & 0x80000000u) | (e > 0 ? ((unsigned)e << 23) | m : 0u));
-  }
-  return top != 0u && top != 0x7FF00000u;
-}
-
-// The same in FP64, where the test compares squares (thr = eps^2 |g|^2, X
-// and x.w = |x_f|^2) and the extremes are kept as bit patterns (integer
-// compares; the FP64 pipe is the kernel's bound).  First a search in FP32 for
-// the face that attains each extreme: |g| scaled to below 2 per component,
-// the FP32 product g . x_f is within 6 2^-24 2 (|x| + |y| + |z|) <= 1.3e-6 |x_f|
-// of the exact one (both operands rounded, three roundings of the sum), so a
-// leader that is 2.6e-6 of the cell's largest |x_f| ahead of every other face
-// and of zero is the FP64 leader, and its FP64 product is the extreme: eight
-// FP64 products per (cell, bin) instead of four per face (with the matrix
-// folded into the weights: 0.85 -> 0.54 ms per launch at 250,047 cells).  Where a lead is
-// smaller (faces that tie by symmetry; a leader within the band of zero) every
-// face's product is formed in FP64.  A component without gradient has no
-// extremes.  at[2q], at[2q + 1]: the first face that attains dpos[q], dneg[q].
-__device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const float4* __restrict__ xf, int k0, int k1,
-                                             const double gr[4][3], const double thr[4], double X, double dpos[4],
-                                             double dneg[4], int at[8]) {
-  float gf[4][3], m1[8], m2[8];
-  bool flat[4], sure = true;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    flat[q] = ((__double_as_longlong(gr[q][0]) | __double_as_longlong(gr[q][1]) | __double_as_longlong(gr[q][2])) &
-               0x7FFFFFFFFFFFFFFFLL) == 0;
-    const bool ok = scaled_f32(gr[q], gf[q]);
-    sure = sure && (ok || flat[q]);
-    m1[2 * q] = m1[2 * q + 1] = m2[2 * q] = m2[2 * q + 1] = 0.0f;
-    at[2 * q] = at[2 * q + 1] = k0;
-  }
-#pragma unroll 2
-  for (int k = k0; k < k1; ++k) {
-    const float4 x = __ldg(xf + k);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float v = gf[q][0] * x.x + gf[q][1] * x.y + gf[q][2] * x.z;
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const float u = h ? -v : v;
-        m2[2 * q + h] = fmaxf(m2[2 * q + h], fminf(m1[2 * q + h], u));
-        at[2 * q + h] = u > m1[2 * q + h] ? k : at[2 * q + h];
-        m1[2 * q + h] = fmaxf(m1[2 * q + h], u);
-      }
-    }
-  }
-  const float lead = 2.6e-6f * sqrtf((float)X);
-#pragma unroll
-  for (int q = 0; q < 4; ++q)
-#pragma unroll
-    for (int h = 0; h < 2; ++h) sure = sure && (flat[q] || m1[2 * q + h] - m2[2 * q + h] > lead);
-  long long bpos[4], bneg[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) bpos[q] = bneg[q] = 0;
-  if (sure) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (flat[q]) continue;
-      const d4 a = xs[at[2 * q]], c = xs[at[2 * q + 1]];
-      bpos[q] = max_bits_pos(0, gr[q][0] * a.x + gr[q][1] * a.y + gr[q][2] * a.z);
-      bneg[q] = max_bits_neg(0, gr[q][0] * c.x + gr[q][1] * c.y + gr[q][2] * c.z);
-    }
-  } else {
-#pragma unroll 1
-    for (int k = k0; k < k1; ++k) {
-      const d4 x = ld4<double>(xs + k);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double dphi = gr[q][0] * x.x + gr[q][1] * x.y + gr[q][2] * x.z;
-        const long long p = max_bits_pos(bpos[q], dphi), n = max_bits_neg(bneg[q], dphi);
-        at[2 * q] = p != bpos[q] ? k : at[2 * q];
-        at[2 * q + 1] = n != bneg[q] ? k : at[2 * q + 1];
-        bpos[q] = p;
-        bneg[q] = n;
-      }
-    }
-  }
-  bool exact = true;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const long long t = __double_as_longlong(thr[q] * X);
-    const double p = __longlong_as_double(bpos[q]), n = neg_from_bits(bneg[q]);
-    exact = exact && (bpos[q] == 0 || __double_as_longlong(p * p) > t) &&
-            (bneg[q] == 0 || __double_as_longlong(n * n) > t);
-  }
-  if (!exact) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) bpos[q] = bneg[q] = 0;
-#pragma unroll 1
-    for (int k = k0; k < k1; ++k) {
-      const d4 x = ld4<double>(xs + k);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double dphi = gr[q][0] * x.x + gr[q][1] * x.y + gr[q][2] * x.z;
-        if (__double_as_longlong(dphi * dphi) > __double_as_longlong(thr[q] * x.w)) {
-          const long long p = max_bits_pos(bpos[q], dphi), n = max_bits_neg(bneg[q], dphi);
-          at[2 * q] = p != bpos[q] ? k : at[2 * q];
-          at[2 * q + 1] = n != bneg[q] ? k : at[2 * q + 1];
-          bpos[q] = p;
-          bneg[q] = n;
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    dpos[q] = __longlong_as_double(bpos[q]);
-    dneg[q] = neg_from_bits(bneg[q]);
   }
 }
 

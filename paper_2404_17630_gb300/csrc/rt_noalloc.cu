@@ -6,65 +6,31 @@
 // own pool, in a real-time loop that must not allocate, or in a plug-in that
 // only receives device pointers.  Such a caller cannot create an rt_ctx
 // (rt_init_mesh allocates), so this entry point takes the whole mesh and state
-// as caller-owned device arrays and keeps its only scratch -- the inverse
-// least-squares matrix of every cell -- in a fixed static device array
-// compiled into the library.
-//
-// The scratch array lives on every GPU that loads the library, until the
-// process exits, and is shared by all calls on that device: each call
-// overwrites the entries of its cells before reading them, so nothing needs
-// clearing, but calls that overlap on the GPU (different streams, or host
-// threads without ordering) race on it.
-//
-// The array's device address is looked up once per device context and
-// cached; when the device's current context changes (a cudaDeviceReset tears
-// the primary context down and the next runtime call creates a new one), the
-// next call looks it up again.
+// as caller-owned device arrays and needs no device memory of its own: a block
+// keeps its cells' geometry in shared memory.
 #include <cstdint>
 #include <cstdio>
-#include <mutex>
+#include <cstring>
 
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include "../../include/rt.h"
+#include "rt_limiter.cuh"
 
 namespace {
 
-constexpr int64_t kNoallocMaxCells = 262144;   // 6 doubles each: 12.6 MB of device memory
+constexpr int64_t kNoallocMaxCells = 262144;
 constexpr int kMaxDevices = 64;
-
-// Host code must not take the address of this array directly: on the host the
-// name is only a stand-in.  The device address comes from cudaGetSymbolAddress.
-__device__ __align__(256) double g_noalloc_minv[6 * kNoallocMaxCells];
-
-std::mutex g_mu;
-double* g_minv_ptr[kMaxDevices] = {};
-void* g_minv_ctx[kMaxDevices] = {};   // the context each cached address belongs to
-
-// cuCtxGetCurrent through the runtime's driver entry point (the library does
-// not link the driver library itself).
-using CtxGetCurrentFn = CUresult (*)(CUcontext*);
-CtxGetCurrentFn ctx_get_current() {
-  static CtxGetCurrentFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      p = nullptr;
-    return (CtxGetCurrentFn)p;
-  }();
-  return fn;
-}
 
 // Kernel launch that returns this launch's own status (a triple-chevron
 // launch only leaves it in the thread's last-error slot, where an error the
 // caller left pending is indistinguishable from it).
 template <class T> struct ident { using type = T; };
 template <class... KA>
-cudaError_t launch(void (*k)(KA...), dim3 grid, dim3 block, cudaStream_t s, typename ident<KA>::type... args) {
+cudaError_t launch(void (*k)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                   typename ident<KA>::type... args) {
   void* p[] = {(void*)&args...};
-  return cudaLaunchKernel((const void*)k, grid, block, p, 0, s);
+  return cudaLaunchKernel((const void*)k, grid, block, p, smem, s);
 }
 
 thread_local char g_err[256];
@@ -74,115 +40,211 @@ rt_status set_err(rt_status st, const char* msg) {
   return st;
 }
 
-__device__ __forceinline__ double mimg(double d, double L) {
-  return L > 0.0 ? __dsub_rn(d, __dmul_rn(L, round(__ddiv_rn(d, L)))) : d;
+using namespace m1rt;
+
+struct NoallocArgs {
+  int C, B;
+  double box;
+  int h_in, h_out, h_two;   // high words of 0.4999, 0.5001 and 1.4999 box (box > 0)
+  int limiter;
+  double lim_eps2;
+  const int32_t *off, *csr, *left, *right;
+  const double *cx, *cy, *cz, *area, *fx, *fy, *fz, *N, *F;
+  double* G;
+  int* bad;
+};
+
+// Minimum image, d - L round(d / L): d itself within 0.4999 L, d -+ L between
+// 0.5001 L and 1.4999 L (told apart by the high words), the expression
+// elsewhere.
+__device__ __forceinline__ double mimg(double d, const NoallocArgs& a) {
+  if (!(a.box > 0.0)) return d;
+  const int hi = __double2hiint(d), h = hi & 0x7FFFFFFF;
+  if (h < a.h_in) return d;
+  if (h > a.h_out && h < a.h_two) return __dsub_rn(d, hi < 0 ? -a.box : a.box);
+  return __dsub_rn(d, __dmul_rn(a.box, round(__ddiv_rn(d, a.box))));
 }
 
-// Inverse of M_i = sum over the cell's faces of A n n^T (n: unit vector to the
-// neighbour's centroid), into the static scratch.
-__global__ void k_noalloc_minv(int C, double box, const int32_t* __restrict__ off, const int32_t* __restrict__ csr,
-                               const int32_t* __restrict__ left, const int32_t* __restrict__ right,
-                               const double* __restrict__ cx, const double* __restrict__ cy,
-                               const double* __restrict__ cz, const double* __restrict__ area, double* minv,
-                               int* bad) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= C) return;
-  double m00 = 0, m01 = 0, m02 = 0, m11 = 0, m12 = 0, m22 = 0;
-  for (int k = off[i]; k < off[i + 1]; ++k) {
-    int e = csr[k], f = e >> 1;
-    int j = (e & 1) ? left[f] : right[f];
-    double d0 = mimg(cx[j] - cx[i], box), d1 = mimg(cy[j] - cy[i], box), d2 = mimg(cz[j] - cz[i], box);
-    double dl = sqrt(d0 * d0 + d1 * d1 + d2 * d2);
-    double n0 = d0 / dl, n1 = d1 / dl, n2 = d2 / dl;
-    double A = area[f];
-    m00 += A * n0 * n0; m01 += A * n0 * n1; m02 += A * n0 * n2;
-    m11 += A * n1 * n1; m12 += A * n1 * n2; m22 += A * n2 * n2;
-  }
-  double c00 = m11 * m22 - m12 * m12, c01 = m12 * m02 - m01 * m22, c02 = m01 * m12 - m11 * m02;
-  double det = m00 * c00 + m01 * c01 + m02 * c02;
-  double* o = minv + 6 * (size_t)i;
-  if (!(det != 0.0) || !isfinite(det)) {
-    atomicExch(bad, 1);
-    for (int q = 0; q < 6; ++q) o[q] = 0.0;
-    return;
-  }
-  o[0] = c00 / det;
-  o[1] = c01 / det;
-  o[2] = c02 / det;
-  o[3] = (m00 * m22 - m02 * m02) / det;
-  o[4] = (m02 * m01 - m00 * m12) / det;
-  o[5] = (m00 * m11 - m01 * m01) / det;
+// Half-edge k of cell i: the weight w = A d / |d|^2 towards the neighbour j and
+// the face-centre offset x with |x|^2.
+struct HalfEdge {
+  d4 w, x;   // w.w: the neighbour id's bits
+};
+__device__ __forceinline__ HalfEdge half_edge(const NoallocArgs& a, int i, int k, double d[3]) {
+  const int e = a.csr[k], f = e >> 1;
+  const int j = (e & 1) ? a.left[f] : a.right[f];
+  const double c0 = a.cx[i], c1 = a.cy[i], c2 = a.cz[i];
+  d[0] = mimg(a.cx[j] - c0, a);
+  d[1] = mimg(a.cy[j] - c1, a);
+  d[2] = mimg(a.cz[j] - c2, a);
+  const double s = div_nr(a.area[f], d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
+  HalfEdge h;
+  h.w = make_d4(s * d[0], s * d[1], s * d[2], id_bits(j, 0.0));
+  const double x0 = mimg(a.fx[f] - c0, a), x1 = mimg(a.fy[f] - c1, a), x2 = mimg(a.fz[f] - c2, a);
+  h.x = make_d4(x0, x1, x2, x0 * x0 + x1 * x1 + x2 * x2);
+  return h;
 }
 
-__device__ __forceinline__ double comp_of(const double* N, const double* Fr, int C, int b, int q, int i) {
-  return q == 0 ? N[(size_t)b * C + i] : Fr[(size_t)(3 * b + q - 1) * C + i];
+__device__ __forceinline__ void add_matrix(const HalfEdge& h, const double d[3], double m[6]) {
+  // A n n^T = w d^T with n = d / |d|
+  m[0] += h.w.x * d[0]; m[1] += h.w.x * d[1]; m[2] += h.w.x * d[2];
+  m[3] += h.w.y * d[1]; m[4] += h.w.y * d[2]; m[5] += h.w.z * d[2];
 }
 
-// Variant of the gradient kernel: the same least-squares sum and slope
-// limiter, with the face weights and face-centre offsets formed on the fly
-// from the caller's geometry and M^-1 read from the static scratch.
-__global__ void k_noalloc_grad(int C, int B, double box, int limiter, double lim_eps2,
-                               const int32_t* __restrict__ off, const int32_t* __restrict__ csr,
-                               const int32_t* __restrict__ left, const int32_t* __restrict__ right,
-                               const double* __restrict__ cx, const double* __restrict__ cy,
-                               const double* __restrict__ cz, const double* __restrict__ area,
-                               const double* __restrict__ fx, const double* __restrict__ fy,
-                               const double* __restrict__ fz, const double* __restrict__ minv,
-                               const double* __restrict__ N, const double* __restrict__ Fr, double* __restrict__ G) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= C * B) return;
-  const int i = t / B, b = t % B;
-  double pi[4], r[4][3], mx[4], mn[4];
-  for (int q = 0; q < 4; ++q) {
-    pi[q] = comp_of(N, Fr, C, b, q, i);
-    r[q][0] = r[q][1] = r[q][2] = 0.0;
-    mx[q] = mn[q] = pi[q];
-  }
-  for (int k = off[i]; k < off[i + 1]; ++k) {
-    const int e = csr[k], f = e >> 1;
-    const int L = left[f], R = right[f];
-    const int j = (e & 1) ? L : R;
-    double d0 = mimg(cx[R] - cx[L], box), d1 = mimg(cy[R] - cy[L], box), d2 = mimg(cz[R] - cz[L], box);
-    double s = area[f] / (d0 * d0 + d1 * d1 + d2 * d2);
-    double w0 = s * d0, w1 = s * d1, w2 = s * d2;
-    for (int q = 0; q < 4; ++q) {
-      double vj = comp_of(N, Fr, C, b, q, j);
-      double dphi = (e & 1) ? (pi[q] - vj) : (vj - pi[q]);
-      r[q][0] += w0 * dphi;
-      r[q][1] += w1 * dphi;
-      r[q][2] += w2 * dphi;
-      mx[q] = vj > mx[q] ? vj : mx[q];
-      mn[q] = vj < mn[q] ? vj : mn[q];
+// A block's cells, and the half-edges it can hold in shared memory: the weight
+// and offset records, the offsets in FP32 and the partial matrices.
+constexpr int kNaCells = 32, kNaCap = 640;
+constexpr size_t kNaSmem = kNaCap * (2 * sizeof(d4) + sizeof(float4)) + kNaCells * 3 * 6 * sizeof(double);
+
+// Least-squares sums and slope limiter, one thread per (cell, bin).  The
+// geometry is formed once per half-edge: the threads of a cell take its
+// half-edges in turn, leave their records in shared memory and add up M =
+// sum A n n^T; each bin then reads the records.  The kernel is bound by the
+// FP64 unit (about 1.7 k FP64 instructions per cell of 15.4 faces and three
+// bins; with the geometry formed per bin and per pass, its divisions and the
+// limiter's quotient per face and component 13 k): 3.22 -> 0.39 ms at 91,125
+// cells.  A block whose cells have
+// more than kNaCap half-edges forms them anew at each use.
+__global__ void __launch_bounds__(kNaCells * 3) k_noalloc_grad(NoallocArgs a) {
+  extern __shared__ __align__(32) unsigned char smem[];
+  d4* sw = reinterpret_cast<d4*>(smem);
+  d4* sx = sw + kNaCap;
+  float4* sf = reinterpret_cast<float4*>(sx + kNaCap);
+  double* sm = reinterpret_cast<double*>(sf + kNaCap);
+  const int B = a.B, C = a.C;
+  const int cl = threadIdx.x / B, b = threadIdx.x - cl * B;
+  const int c0 = blockIdx.x * kNaCells, c1 = min(c0 + kNaCells, C), i = c0 + cl;
+  const int kb = a.off[c0], n = a.off[c1] - kb;
+  const bool act = i < c1, staged = n <= kNaCap;
+  const int k0 = act ? a.off[i] : 0, k1 = act ? a.off[i + 1] : 0;
+  double m[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, d[3];
+  if (staged) {
+    for (int k = k0 + b; k < k1; k += B) {
+      const HalfEdge h = half_edge(a, i, k, d);
+      add_matrix(h, d, m);
+      sw[k - kb] = h.w;
+      sx[k - kb] = h.x;
+      sf[k - kb] = make_float4((float)h.x.x, (float)h.x.y, (float)h.x.z, 0.f);
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) sm[threadIdx.x * 6 + q] = m[q];
+    __syncthreads();
+    if (!act) return;
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      m[q] = sm[cl * B * 6 + q];
+      for (int p = 1; p < B; ++p) m[q] += sm[(cl * B + p) * 6 + q];
+    }
+  } else {
+    if (!act) return;
+    for (int k = k0; k < k1; ++k) {
+      const HalfEdge h = half_edge(a, i, k, d);
+      add_matrix(h, d, m);
     }
   }
-  const double* m = minv + 6 * (size_t)i;
-  double g[4][3], gg[4], psi[4];
+  // inverse of M
+  const double v00 = m[3] * m[5] - m[4] * m[4], v01 = m[4] * m[2] - m[1] * m[5], v02 = m[1] * m[4] - m[3] * m[2];
+  const double det = m[0] * v00 + m[1] * v01 + m[2] * v02;
+  double* Go = a.G + ((size_t)i * B + b) * 12;
+  if (!(det != 0.0) || !isfinite(det)) {
+    atomicExch(a.bad, 1);
+#pragma unroll
+    for (int q = 0; q < 12; ++q) Go[q] = 0.0;
+    return;
+  }
+  const double idet = 1.0 / det;
+  const double i00 = v00 * idet, i01 = v01 * idet, i02 = v02 * idet, i11 = (m[0] * m[5] - m[2] * m[2]) * idet,
+               i12 = (m[2] * m[1] - m[0] * m[4]) * idet, i22 = (m[0] * m[3] - m[1] * m[1]) * idet;
+  const double* f[4] = {a.N + (size_t)b * C, a.F + (size_t)(3 * b) * C, a.F + (size_t)(3 * b + 1) * C,
+                        a.F + (size_t)(3 * b + 2) * C};
+  double pi[4], r[4][3];
+  long long up[4], dn[4];   // largest and most negative difference to a neighbour, as bits
+#pragma unroll
   for (int q = 0; q < 4; ++q) {
-    g[q][0] = m[0] * r[q][0] + m[1] * r[q][1] + m[2] * r[q][2];
-    g[q][1] = m[1] * r[q][0] + m[3] * r[q][1] + m[4] * r[q][2];
-    g[q][2] = m[2] * r[q][0] + m[4] * r[q][1] + m[5] * r[q][2];
-    gg[q] = g[q][0] * g[q][0] + g[q][1] * g[q][1] + g[q][2] * g[q][2];
+    pi[q] = f[q][i];
+    r[q][0] = r[q][1] = r[q][2] = 0.0;
+    up[q] = dn[q] = 0;
+  }
+  long long X = 0;          // largest |x_f|^2
+  for (int k = k0; k < k1; ++k) {
+    HalfEdge h;
+    if (staged) {
+      h.w = sw[k - kb];
+      h.x = sx[k - kb];
+    } else {
+      h = half_edge(a, i, k, d);
+    }
+    const int j = bits_id(h.w.w);
+    X = __double_as_longlong(h.x.w) > X ? __double_as_longlong(h.x.w) : X;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double dphi = f[q][j] - pi[q];
+      r[q][0] += h.w.x * dphi;
+      r[q][1] += h.w.y * dphi;
+      r[q][2] += h.w.z * dphi;
+      up[q] = max_bits_pos(up[q], dphi);
+      dn[q] = max_bits_neg(dn[q], dphi);
+    }
+  }
+  double g[4][3], thr[4], psi[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    g[q][0] = i00 * r[q][0] + i01 * r[q][1] + i02 * r[q][2];
+    g[q][1] = i01 * r[q][0] + i11 * r[q][1] + i12 * r[q][2];
+    g[q][2] = i02 * r[q][0] + i12 * r[q][1] + i22 * r[q][2];
+    thr[q] = a.lim_eps2 * (g[q][0] * g[q][0] + g[q][1] * g[q][1] + g[q][2] * g[q][2]);
     psi[q] = 1.0;
   }
-  if (limiter) {
-    for (int k = off[i]; k < off[i + 1]; ++k) {
-      const int f = csr[k] >> 1;
-      double x0 = mimg(fx[f] - cx[i], box), x1 = mimg(fy[f] - cy[i], box), x2 = mimg(fz[f] - cz[i], box);
-      double xx = x0 * x0 + x1 * x1 + x2 * x2;
+  if (a.limiter) {
+    double dpos[4], dneg[4];
+    if (staged) {
+      int at[8];
+      lim_extremes(sx, sf, k0 - kb, k1 - kb, g, thr, __longlong_as_double(X), dpos, dneg, at);
+    } else {
+      long long p[4] = {0, 0, 0, 0}, q4[4] = {0, 0, 0, 0};
+      for (int k = k0; k < k1; ++k) {
+        const d4 x = half_edge(a, i, k, d).x;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const double dphi = g[q][0] * x.x + g[q][1] * x.y + g[q][2] * x.z;
+          if (__double_as_longlong(dphi * dphi) > __double_as_longlong(thr[q] * x.w)) {
+            p[q] = max_bits_pos(p[q], dphi);
+            q4[q] = max_bits_neg(q4[q], dphi);
+          }
+        }
+      }
+#pragma unroll
       for (int q = 0; q < 4; ++q) {
-        double dphi = g[q][0] * x0 + g[q][1] * x1 + g[q][2] * x2;
-        double lim = 1.0;
-        if (dphi * dphi > lim_eps2 * gg[q] * xx) lim = dphi > 0 ? (mx[q] - pi[q]) / dphi : (mn[q] - pi[q]) / dphi;
-        psi[q] = lim < psi[q] ? lim : psi[q];
+        dpos[q] = __longlong_as_double(p[q]);
+        dneg[q] = neg_from_bits(q4[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      // the smallest quotient is the one by the largest g . x: rounded division
+      // is monotone in the divisor
+      if (gt_nonneg(dpos[q], 0.0)) {
+        const double lim = div_nr(__longlong_as_double(up[q]), dpos[q]);
+        psi[q] = gt_nonneg(psi[q], lim) ? lim : psi[q];
+      }
+      if (__double_as_longlong(dneg[q]) != 0) {
+        const double lim = div_nr(neg_from_bits(dn[q]), dneg[q]);
+        psi[q] = gt_nonneg(psi[q], lim) ? lim : psi[q];
       }
     }
   }
-  double* Go = G + (size_t)t * 12;
+#pragma unroll
   for (int q = 0; q < 4; ++q) {
     Go[3 * q + 0] = g[q][0] * psi[q];
     Go[3 * q + 1] = g[q][1] * psi[q];
     Go[3 * q + 2] = g[q][2] * psi[q];
   }
+}
+
+int high_word(double v) {
+  uint64_t b;
+  std::memcpy(&b, &v, sizeof b);
+  return (int)(b >> 32);
 }
 
 // Device memory of the current device `dev`, or managed memory.  Device memory
@@ -225,26 +287,6 @@ rt_status rt_gradients_noalloc(const rt_cells* cells, const rt_faces* faces, con
   for (const void* p : dev_ptrs)
     if (!p || !on_device(p, dev))
       return set_err(RT_INVALID_ARG, "rt_gradients_noalloc: every array must be device memory of the current device");
-  double* minv = nullptr;
-  {
-    std::lock_guard<std::mutex> lk(g_mu);
-    CUcontext cur = nullptr;
-    CtxGetCurrentFn get = ctx_get_current();
-    if (get && get(&cur) != CUDA_SUCCESS) cur = nullptr;
-    if (!g_minv_ptr[dev] || (cur && cur != (CUcontext)g_minv_ctx[dev])) {
-      // first call on this device, or its context was replaced: look the
-      // address up with this device current
-      void* p = nullptr;
-      cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_minv);
-      if (e != cudaSuccess || !p) {
-        cudaGetLastError();
-        return set_err(RT_CUDA, "rt_gradients_noalloc: cudaGetSymbolAddress failed");
-      }
-      g_minv_ptr[dev] = (double*)p;
-      g_minv_ctx[dev] = (void*)cur;
-    }
-    minv = g_minv_ptr[dev];
-  }
   cudaStream_t s = (cudaStream_t)stream;
   const int Ci = (int)C;
   if (order < 2) {
@@ -259,15 +301,17 @@ rt_status rt_gradients_noalloc(const rt_cells* cells, const rt_faces* faces, con
     cudaGetLastError();
     return set_err(RT_CUDA, "rt_gradients_noalloc: memset failed");
   }
-  const int t = 256;
-  cudaError_t e = launch(k_noalloc_minv, dim3((Ci + t - 1) / t), dim3(t), s, Ci, box, cell_off, cell_faces,
-                         faces->left, faces->right, cells->cx, cells->cy, cells->cz, faces->area, minv, bad_cell);
-  if (e == cudaSuccess) {
-    const long long n = (long long)C * n_bins;
-    e = launch(k_noalloc_grad, dim3((unsigned)((n + t - 1) / t)), dim3(t), s, Ci, n_bins, box, limiter,
-               lim_eps * lim_eps, cell_off, cell_faces, faces->left, faces->right, cells->cx, cells->cy, cells->cz,
-               faces->area, faces->fx, faces->fy, faces->fz, (const double*)minv, N, F_red, G);
-  }
+  NoallocArgs a{};
+  a.C = Ci; a.B = n_bins; a.box = box;
+  a.h_in = high_word(0.4999 * box); a.h_out = high_word(0.5001 * box); a.h_two = high_word(1.4999 * box);
+  a.limiter = limiter; a.lim_eps2 = lim_eps * lim_eps;
+  a.off = cell_off; a.csr = cell_faces; a.left = faces->left; a.right = faces->right;
+  a.cx = cells->cx; a.cy = cells->cy; a.cz = cells->cz; a.area = faces->area;
+  a.fx = faces->fx; a.fy = faces->fy; a.fz = faces->fz; a.N = N; a.F = F_red; a.G = G; a.bad = bad_cell;
+  cudaError_t e = cudaFuncSetAttribute(k_noalloc_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNaSmem);
+  if (e == cudaSuccess)
+    e = launch(k_noalloc_grad, dim3((unsigned)((Ci + kNaCells - 1) / kNaCells)), dim3(kNaCells * n_bins), kNaSmem,
+               s, a);
   if (e != cudaSuccess) {
     cudaGetLastError();   // the failed launch's own error
     return set_err(RT_CUDA, cudaGetErrorString(e));
