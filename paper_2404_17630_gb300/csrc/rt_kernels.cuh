@@ -1087,9 +1087,13 @@ __global__ void k_reciprocal(int n, const double* __restrict__ in, double* out) 
 
 // A worklist of at most this many cells goes to groups of lanes (rest_groups),
 // a longer one to one thread per cell (rest_threads): a group's attempt has a
-// fraction of the latency but costs the FP64 unit several times as much per
-// cell.
-constexpr int kGroupMax = 4096;
+// third (FP64) or half (mixed) of the latency, but costs the FP64 unit several
+// times as much per cell, so that groups win while the longest chains decide.
+// Far from equilibrium (mean chain 11-47 attempts, longest 150-360), ms by
+// threads / by groups: FP64 4.2 / 1.3 at 991 cells, 5.7 / 2.4 at 12,035,
+// 8.8 / 6.2 at 32,006, 10.8 / 9.4 at 61,427; mixed 0.94 / 0.58, 1.29 / 0.98,
+// 1.89 / 1.90, 2.28 / 2.87.
+constexpr int kGroupMax64 = 49152, kGroupMaxMixed = 24576;
 
 // Worklist of the cells whose first attempt was rejected.
 struct ChemWork {
@@ -1317,7 +1321,7 @@ __global__ void __launch_bounds__(128) k_chem_rest(CellArgs a, ChemParams P, flo
                                                    ChemWork w) {
   const int total = *(volatile int*)w.ctl;
   if (total == 0) return;   // nothing was rejected: the worklist's counters are all zero already
-  if (total <= kGroupMax) rest_groups(a, P, shadow, w, total);
+  if (total <= kGroupMaxMixed) rest_groups(a, P, shadow, w, total);
   else rest_threads(a, P, shadow, w, total);
   rest_done(w.ctl);
 }
@@ -1620,7 +1624,7 @@ __global__ void __launch_bounds__(128) k_chem64_rest(CellArgs a, ChemParams P, c
                                                      ChemTape tape) {
   const int total = *(volatile int*)work_ctl;
   if (total == 0) return;   // nothing was rejected: the worklist's counters are all zero already
-  if (total <= kGroupMax) rest_groups64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, total);
+  if (total <= kGroupMax64) rest_groups64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, total);
   else rest_threads64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, total);
   rest_done(work_ctl);
 }

@@ -1,9 +1,10 @@
-"""The chemistry's worklist on either side of the length where it changes from
-groups of lanes to one thread per cell (4096 rejected cells): far from
-equilibrium almost every cell's first attempt is rejected, so the 15^3 and
-17^3 meshes lie below and above it; 1, 2 and 3 bins, thermal and isothermal, a
-hydrogen-only gas and rates switched off.  Bounds as in the parity tests: FP64
-1e-12 with the oracle's substep counts, mixed 1e-4."""
+"""The chemistry's worklist by groups of lanes and by one thread per cell, which
+take over at 49,152 (FP64) and 24,576 (mixed) rejected cells: far from
+equilibrium almost every cell's first attempt is rejected, so the 28^3 and 30^3
+meshes (mixed) and the 36^3 and 37^3 meshes (FP64) lie below and above; 1, 2 and 3
+bins, thermal and isothermal, a hydrogen-only gas and rates switched off on
+small meshes.  Bounds as in the parity tests: FP64 1e-12 with the oracle's
+substep counts, mixed 1e-4."""
 import numpy as np
 import pytest
 
@@ -50,3 +51,11 @@ def test_worklist_mixed(n, kw):
     err, ns, ref = _run(n, "mixed", **kw)
     assert err < 1e-4
     assert (ns >= 1).all()
+
+
+@pytest.mark.parametrize("prec,n", [("fp64", 36), ("fp64", 37), ("mixed", 28), ("mixed", 30)])
+def test_worklist_lengths(prec, n):
+    err, ns, ref = _run(n, prec)
+    assert err < (1e-12 if prec == "fp64" else 1e-4)
+    if prec == "fp64":
+        assert np.array_equal(ns, ref)
