@@ -169,7 +169,8 @@ template <> Geo<float> geo<float>(const rt_ctx* c) {
                     c->n_act_faces};
 }
 
-ChemParams chem_params(const rt_ctx* ctx) {
+// dt: the length of the first attempts
+ChemParams chem_params(const rt_ctx* ctx, double dt) {
   ChemParams P;
   const rt_config& c = ctx->cfg;
   P.B = c.n_bins;
@@ -190,6 +191,11 @@ ChemParams chem_params(const rt_ctx* ctx) {
       if (P.eps[b][s] != 0.0) P.emask |= 1 << (3 * b + s);
       P.heat_f[b][s] = (float)(P.eps[b][s] * P.sigma[b][s] / kHeatScale);
     }
+  P.cdt = c.c_red * dt;
+  for (int b = 0; b < kMaxBins; ++b)
+    for (int s = 0; s < 3; ++s) P.csig[b][s] = P.cdt * P.sigma[b][s];
+  P.cdt_heat = (float)(P.cdt * kHeatScale);
+  P.dt_cool = (float)(dt * kCoolScale);
   return P;
 }
 
@@ -326,7 +332,7 @@ void launch_gather(rt_ctx* ctx, double dt, int stage = 0) {
 void launch_chem(rt_ctx* ctx, double dt, const ChemTape* tape = nullptr) {
   ProfScope ps(ctx, RT_KERNEL_CHEM);
   CellArgs a = cell_args(ctx, dt, 0, 1, 1);
-  ChemParams P = chem_params(ctx);
+  ChemParams P = chem_params(ctx, dt);
   const int t = 128;
   const int nc = ctx->all_active ? ctx->C : ctx->n_act;
   if (nc == 0) return;
@@ -1240,7 +1246,7 @@ rt_status adj_subcycle(rt_ctx* ctx, int slot, double dts) {
   const d4* pc_rad = A.tp_rad_chem + slot * C * B;
   const double* pc_x5 = A.tp_x5 + slot * 5 * C;
   const double* pc_T = A.tp_T + slot * C;
-  ChemParams P = chem_params(ctx);
+  ChemParams P = chem_params(ctx, dts);
   ChemAdjArgs ca = chem_adj_args(ctx, pc_rad, pc_x5, pc_T, dts);
   ca.last = A.tape_last + (size_t)slot * C;
   ca.lin = (const AttemptLin*)A.lin;

@@ -23,6 +23,10 @@ struct ChemParams {
   int smask;         // bit 3b+s: sigma[b][s] != 0
   int emask;         // bit 3b+s: eps[b][s] != 0
   float heat_f[kMaxBins][3];   // mixed precision: eps sigma / kHeatScale in FP32
+  // for the first attempts, whose length dt is the same for every cell:
+  // c_red dt, c_red dt sigma, and the scaled factors of the heat and cooling
+  double cdt, csig[kMaxBins][3];
+  float cdt_heat, dt_cool;
 };
 
 // Scale of the FP32 photoheating products: eps sigma (~1e-29 erg cm^2) is
@@ -316,12 +320,16 @@ struct GasState {
   double xHI, xHII, yI, yII, yIII, T;
 };
 
+// IntCvt (the first attempt, over the common length): c dt sigma comes with
+// the kernel's arguments instead of being multiplied out in the optical
+// depths, the photoionisation rates and the photon removal: 96 FP64
+// instructions per attempt instead of 109, of which the first pass is made.
 template <bool IntCvt>
 __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double dt, const GasState& s,
                                          GasState& t, float sc_out[kMaxBins]) {
   const int B = P.B;
-  const double c = P.c_red;
-  const double cdt = c * dt;
+  const double cdt = IntCvt ? P.cdt : P.c_red * dt;
+  auto sg = [&](int b, int sp) { return IntCvt ? P.csig[b][sp] : P.sigma[b][sp]; };
   const double nHe = P.y_he * nH;
   const bool recomb = P.flags & 1, coll = P.flags & 2, cool = P.flags & 4, heat = P.flags & 8;
   // rate coefficients and their products with n_e in FP32 (the fits carry
@@ -336,24 +344,26 @@ __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double 
 #pragma unroll
   for (int b = 0; b < kMaxBins; ++b) {
     if (b < B) {
-      double kap = 0.0;
+      double kap = IntCvt ? 1.0 : 0.0;
 #pragma unroll
       for (int sp = 0; sp < 3; ++sp)
-        if (P.smask & (1 << (3 * b + sp))) kap = fma(P.sigma[b][sp], ns[sp], kap);
-      inv1pt[b] = rcp64<IntCvt>(fma(cdt, kap, 1.0));
+        if (P.smask & (1 << (3 * b + sp))) kap = fma(sg(b, sp), ns[sp], kap);
+      inv1pt[b] = rcp64<IntCvt>(IntCvt ? kap : fma(cdt, kap, 1.0));
       Nbar[b] = s.N[b] * inv1pt[b];
 #pragma unroll
       for (int sp = 0; sp < 3; ++sp)
-        if (P.smask & (1 << (3 * b + sp))) Gs[sp] = fma(P.sigma[b][sp], Nbar[b], Gs[sp]);
+        if (P.smask & (1 << (3 * b + sp))) Gs[sp] = fma(sg(b, sp), Nbar[b], Gs[sp]);
     }
   }
-  const double G0 = Gs[0], G1 = Gs[1], G2 = Gs[2];
+  // photoionisations over the attempt: c dt times the sums
+  const double G0 = IntCvt ? Gs[0] : cdt * Gs[0], G1 = IntCvt ? Gs[1] : cdt * Gs[1],
+               G2 = IntCvt ? Gs[2] : cdt * Gs[2];
   // n_e enters only the FP32 products with the rate coefficients (and the
   // FP32 cooling): formed in FP32 from the FP32 images of the densities
   const float nHf = to_f<IntCvt>(nH), nHef = to_f<IntCvt>(nHe);
   const float ne_he = nHef * fmaf(2.0f, to_f<IntCvt>(s.yIII), to_f<IntCvt>(s.yII));
   const float ne0f = fmaf(nHf, to_f<IntCvt>(s.xHII), ne_he);
-  const double aH = coll ? fma(dt, to_d<IntCvt>(r.bHI * ne0f), cdt * G0) : cdt * G0;
+  const double aH = coll ? fma(dt, to_d<IntCvt>(r.bHI * ne0f), G0) : G0;
   const double bH = recomb ? dt * to_d<IntCvt>(r.aHII * ne0f) : 0.0;
   const double iden = rcp64<IntCvt>(1.0 + aH + bH);
   // backward Euler for (x_HI, x_HII): x_HI' = (x_HI + bH (x_HI + x_HII)) / (1
@@ -363,9 +373,9 @@ __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double 
   t.xHI = fma(bH, xs, s.xHI) * iden;
   t.xHII = fma(aH, xs, s.xHII) * iden;
   const float ne1f = fmaf(nHf, to_f<IntCvt>(t.xHII), ne_he);
-  const double A = coll ? fma(dt, to_d<IntCvt>(r.bHeI * ne1f), cdt * G1) : cdt * G1;
+  const double A = coll ? fma(dt, to_d<IntCvt>(r.bHeI * ne1f), G1) : G1;
   const double Bb = recomb ? dt * to_d<IntCvt>(r.aHeII * ne1f) : 0.0;
-  const double Cc = coll ? fma(dt, to_d<IntCvt>(r.bHeII * ne1f), cdt * G2) : cdt * G2;
+  const double Cc = coll ? fma(dt, to_d<IntCvt>(r.bHeII * ne1f), G2) : G2;
   const double D = recomb ? dt * to_d<IntCvt>(r.aHeIII * ne1f) : 0.0;
   const double iA = rcp64<IntCvt>(1.0 + A), iD = rcp64<IntCvt>(1.0 + D);
   t.yII = (s.yII + A * s.yI * iA + D * s.yIII * iD) * rcp64<IntCvt>(1.0 + Bb * iA + Cc * iD);
@@ -387,8 +397,8 @@ __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double 
       double suma = 0.0;
 #pragma unroll
       for (int sp = 0; sp < 3; ++sp)
-        if (P.smask & (1 << (3 * b + sp))) suma = fma(P.sigma[b][sp], m[sp], suma);
-      const double taup = cdt * suma;
+        if (P.smask & (1 << (3 * b + sp))) suma = fma(sg(b, sp), m[sp], suma);
+      const double taup = IntCvt ? suma : cdt * suma;
       double sc = fma(-taup, inv1pt[b], 1.0);
       // sc <- max(sc, 0) on the integer pipe (a double's bits order like
       // the value where it is positive)
@@ -416,7 +426,9 @@ __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double 
       lam_s = RateEval<true>::template cooling_scaled<IntCvt>(s.T, ne0f, nHf * to_f<IntCvt>(s.xHI), nHf * to_f<IntCvt>(s.xHII),
                                              nHef * to_f<IntCvt>(s.yI), nHef * to_f<IntCvt>(s.yII), nHef * to_f<IntCvt>(s.yIII));
     }
-    const float de = fmaf(heat ? to_f<IntCvt>(cdt * kHeatScale) : 0.0f, hsum, -(to_f<IntCvt>(dt * kCoolScale) * lam_s));
+    const float hs = IntCvt ? P.cdt_heat : to_f<IntCvt>(cdt * kHeatScale);
+    const float cs = IntCvt ? P.dt_cool : to_f<IntCvt>(dt * kCoolScale);
+    const float de = fmaf(heat ? hs : 0.0f, hsum, -(cs * lam_s));
     // the change of n_e from the FP64 differences of the fractions (they
     // cancel), combined in FP32
     const float dnef = fmaf(nHf, to_f<IntCvt>(t.xHII - s.xHII),
