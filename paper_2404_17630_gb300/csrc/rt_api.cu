@@ -119,6 +119,17 @@ bool is_device_ptr(const void* p) {
   return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// p can be read and written by the context's kernels as doubles: plain device
+// memory of its own device (not managed, not a peer's), aligned.
+bool direct_ptr(const rt_ctx* ctx, const void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == ctx->device && ((uintptr_t)p & 7) == 0;
+}
+
 // Copy n elements from caller memory (host or device) to device memory dst.
 rt_status copy_in(rt_ctx* ctx, void* dst, const void* src, size_t bytes) {
   cudaMemcpyKind k = is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
@@ -377,17 +388,21 @@ void transport(rt_ctx* ctx, double dt) {
   launch_gather(ctx, dt, 2);
 }
 
-// Mixed precision: the state (radN, FP32 sweep records) from the interface
-// records in ctx->rad, and back.
-void refresh_shadow(rt_ctx* ctx) {
-  if (!mixed(ctx)) return;
-  long long n = (long long)ctx->C * ctx->B;
-  k_split_rad<<<nblk(n), kThreads, 0, ctx->stream>>>((int)n, ctx->rad, ctx->radN, ctx->shadow);
+// The radiation state from component-major device arrays (F may be null), and
+// back (either may be null).
+void pack_state(rt_ctx* ctx, const double* N, const double* F) {
+  const double ic = 1.0 / ctx->cfg.c_red;
+  if (mixed(ctx))
+    k_pack_mixed<<<nblk(ctx->C), kThreads, 0, ctx->stream>>>(ctx->C, ctx->B, ic, N, F, ctx->radN, ctx->shadow);
+  else
+    k_pack_rad<<<nblk(ctx->C), kThreads, 0, ctx->stream>>>(ctx->C, ctx->B, ic, N, F, ctx->rad);
 }
-void join_state(rt_ctx* ctx) {
-  if (!mixed(ctx)) return;
-  long long n = (long long)ctx->C * ctx->B;
-  k_join_rad<<<nblk(n), kThreads, 0, ctx->stream>>>((int)n, ctx->radN, ctx->shadow, ctx->rad);
+void unpack_state(rt_ctx* ctx, double* N, double* F) {
+  const double c = ctx->cfg.c_red;
+  if (mixed(ctx))
+    k_unpack_mixed<<<nblk(ctx->C), kThreads, 0, ctx->stream>>>(ctx->C, ctx->B, c, ctx->radN, ctx->shadow, N, F);
+  else
+    k_unpack_rad<<<nblk(ctx->C), kThreads, 0, ctx->stream>>>(ctx->C, ctx->B, c, ctx->rad, N, F);
 }
 
 rt_status launched(rt_ctx* ctx, const char* what) {
@@ -524,7 +539,8 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   AL(ctx->off, C + 1); AL(ctx->csr, 2 * (size_t)F); AL(ctx->nbr, 2 * (size_t)F); AL(ctx->lr, F);
   AL(ctx->nA64, F); AL(ctx->rL64, F); AL(ctx->rR64, F); AL(ctx->w64, F); AL(ctx->minv64, 6 * (size_t)C);
   if (ctx->cfg.time_order == 2) AL(ctx->rad0, (size_t)C * B);
-  AL(ctx->rad, (size_t)C * B); AL(ctx->nH, C); AL(ctx->x5, 5 * (size_t)C); AL(ctx->T, C);
+  if (!mixed(ctx)) AL(ctx->rad, (size_t)C * B);
+  AL(ctx->nH, C); AL(ctx->x5, 5 * (size_t)C); AL(ctx->T, C);
   AL(ctx->src_idx, C); AL(ctx->nsub, C); AL(ctx->status, 1);
   ctx->stage_n = std::max<size_t>(4 * (size_t)B * C, 7 * (size_t)F);
   ctx->stage_n = std::max<size_t>(ctx->stage_n, 5 * (size_t)C);
@@ -619,7 +635,12 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   CK(cudaStreamSynchronize(ctx->stream), "geometry");
   if (h_status & kStSingular) return fail(ctx, RT_BAD_MESH, "singular least-squares matrix (degenerate cell)");
   // default state: no radiation, neutral gas at 1e4 K, no sources
-  CK(cudaMemsetAsync(ctx->rad, 0, (size_t)C * B * sizeof(d4), ctx->stream), "state");
+  if (mx) {
+    CK(cudaMemsetAsync(ctx->radN, 0, (size_t)C * B * 8, ctx->stream), "state");
+    CK(cudaMemsetAsync(ctx->shadow, 0, (size_t)C * B * sizeof(float4), ctx->stream), "state");
+  } else {
+    CK(cudaMemsetAsync(ctx->rad, 0, (size_t)C * B * sizeof(d4), ctx->stream), "state");
+  }
   CK(cudaMemsetAsync(ctx->nH, 0, (size_t)C * 8, ctx->stream), "state");
   CK(cudaMemsetAsync(ctx->nsub, 0, (size_t)C * 4, ctx->stream), "state");
   CK(cudaMemsetAsync(ctx->src_idx, 0xff, (size_t)C * 4, ctx->stream), "state");
@@ -632,8 +653,6 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
     CK(cudaStreamSynchronize(ctx->stream), "state");
   }
   ctx->n_src_cells = 0;
-  refresh_shadow(ctx);
-  if ((st = launched(ctx, "state init"))) return st;
   ctx->mesh_ready = true;
   return RT_OK;
 }
@@ -654,13 +673,16 @@ rt_status rt_set_radiation(rt_ctx* ctx, const double* N, const double* F) {
   if (st) return st;
   if (!N) return fail(ctx, RT_INVALID_ARG, "N is NULL");
   const size_t C = ctx->C, B = ctx->B;
-  double* sN = ctx->stage;
-  double* sF = ctx->stage + B * C;
-  if ((st = copy_in(ctx, sN, N, B * C * 8))) return st;
-  if (F && (st = copy_in(ctx, sF, F, 3 * B * C * 8))) return st;
-  k_pack_rad<<<nblk((long long)B * C), kThreads, 0, ctx->stream>>>((int)C, (int)B, 1.0 / ctx->cfg.c_red, sN,
-                                                                   F ? sF : nullptr, ctx->rad);
-  refresh_shadow(ctx);
+  const double *dN = N, *dF = F;
+  if (!direct_ptr(ctx, N) || (F && !direct_ptr(ctx, F))) {
+    double* sN = ctx->stage;
+    double* sF = ctx->stage + B * C;
+    if ((st = copy_in(ctx, sN, N, B * C * 8))) return st;
+    if (F && (st = copy_in(ctx, sF, F, 3 * B * C * 8))) return st;
+    dN = sN;
+    dF = F ? sF : nullptr;
+  }
+  pack_state(ctx, dN, dF);
   return launched(ctx, "set radiation");
 }
 
@@ -927,20 +949,23 @@ rt_status rt_get_fields(rt_ctx* ctx, uint32_t mask, double* const* out) {
   const size_t C = ctx->C, B = ctx->B;
   int k = 0;
   if (mask & (RT_FIELD_N | RT_FIELD_F)) {
-    double* sN = ctx->stage;
-    double* sF = ctx->stage + B * C;
-    join_state(ctx);
-    k_unpack_rad<<<nblk((long long)B * C), kThreads, 0, ctx->stream>>>((int)C, (int)B, ctx->cfg.c_red, ctx->rad,
-                                                                        sN, sF);
-    if ((st = launched(ctx, "get fields"))) return st;
+    double *oN = nullptr, *oF = nullptr;
     if (mask & RT_FIELD_N) {
       if (!out[k]) return fail(ctx, RT_INVALID_ARG, "output %d is NULL", k);
-      if ((st = copy_out(ctx, out[k++], sN, B * C * 8))) return st;
+      oN = out[k++];
     }
     if (mask & RT_FIELD_F) {
       if (!out[k]) return fail(ctx, RT_INVALID_ARG, "output %d is NULL", k);
-      if ((st = copy_out(ctx, out[k++], sF, 3 * B * C * 8))) return st;
+      oF = out[k++];
     }
+    // straight into the caller's device arrays, or through the staging buffer
+    const bool dN = oN && direct_ptr(ctx, oN), dF = oF && direct_ptr(ctx, oF);
+    double* sN = !oN ? nullptr : (dN ? oN : ctx->stage);
+    double* sF = !oF ? nullptr : (dF ? oF : ctx->stage + B * C);
+    unpack_state(ctx, sN, sF);
+    if ((st = launched(ctx, "get fields"))) return st;
+    if (oN && !dN && (st = copy_out(ctx, oN, sN, B * C * 8))) return st;
+    if (oF && !dF && (st = copy_out(ctx, oF, sF, 3 * B * C * 8))) return st;
   }
   if (mask & RT_FIELD_X) {
     if (!out[k]) return fail(ctx, RT_INVALID_ARG, "output %d is NULL", k);
@@ -952,11 +977,8 @@ rt_status rt_get_fields(rt_ctx* ctx, uint32_t mask, double* const* out) {
   }
   if (mask & RT_FIELD_NSUB) {
     if (!out[k]) return fail(ctx, RT_INVALID_ARG, "output %d is NULL", k);
-    std::vector<int32_t> h(C);
-    CK(cudaMemcpyAsync(h.data(), ctx->nsub, C * 4, cudaMemcpyDeviceToHost, ctx->stream), "nsub");
-    CK(cudaStreamSynchronize(ctx->stream), "nsub");
-    std::vector<double> d(h.begin(), h.end());
-    if ((st = copy_in(ctx, ctx->stage, d.data(), C * 8))) return st;
+    k_widen<<<nblk((long long)C), kThreads, 0, ctx->stream>>>((int)C, ctx->nsub, ctx->stage);
+    if ((st = launched(ctx, "get fields"))) return st;
     if ((st = copy_out(ctx, out[k++], ctx->stage, C * 8))) return st;
   }
   CK(cudaStreamSynchronize(ctx->stream), "get fields");
@@ -1378,7 +1400,7 @@ rt_status rt_adjoint(rt_ctx* ctx, double dt, int n_sub, int checkpoint_every, co
   if (lam_N && (st = copy_in(ctx, sN, lam_N, B * C * 8))) return st;
   if (lam_F && (st = copy_in(ctx, sF, lam_F, 3 * B * C * 8))) return st;
   // dL/d(F/c) = c dL/dF
-  k_pack_rad<<<nblk((long long)B * C), kThreads, 0, ctx->stream>>>((int)C, (int)B, ctx->cfg.c_red, sN, sF, A.lam_rad);
+  k_pack_rad<<<nblk((long long)C), kThreads, 0, ctx->stream>>>((int)C, (int)B, ctx->cfg.c_red, sN, sF, A.lam_rad);
   CK(cudaMemsetAsync(A.lam_x5, 0, 5 * C * 8, ctx->stream), "adjoint");
   CK(cudaMemsetAsync(A.lam_T, 0, C * 8, ctx->stream), "adjoint");
   if (lam_x5 && (st = copy_in(ctx, A.lam_x5, lam_x5, 5 * C * 8))) return st;
@@ -1411,7 +1433,7 @@ rt_status rt_adjoint(rt_ctx* ctx, double dt, int n_sub, int checkpoint_every, co
   }
   if (dL_dnH && (st = copy_out(ctx, dL_dnH, A.lam_nH, C * 8))) return st;
   if (lam0_N || lam0_F) {
-    k_unpack_rad<<<nblk((long long)B * C), kThreads, 0, ctx->stream>>>((int)C, (int)B, 1.0 / ctx->cfg.c_red,
+    k_unpack_rad<<<nblk((long long)C), kThreads, 0, ctx->stream>>>((int)C, (int)B, 1.0 / ctx->cfg.c_red,
                                                                         A.lam_rad, sN, sF);
     if (lam0_N && (st = copy_out(ctx, lam0_N, sN, B * C * 8))) return st;
     if (lam0_F && (st = copy_out(ctx, lam0_F, sF, 3 * B * C * 8))) return st;

@@ -34,7 +34,7 @@ struct rt_ctx {
   f8* fa32 = nullptr;          // FP32 face records (n, A, x_f - s_L, left)
   float4* fb32 = nullptr;      // FP32 face records (x_f - s_R, right)
   // state
-  d4* rad = nullptr;      // [C][B] (N, F / c): the FP64 state; mixed precision: the interface records only
+  d4* rad = nullptr;      // FP64 path: [C][B] (N, F / c)
   double* radN = nullptr;      // mixed precision: N [C][B] in FP64
   float4* shadow = nullptr;    // mixed precision: FP32 sweep records [C][B] (N rounded, F / c: the flux state)
   double *nH = nullptr, *x5 = nullptr, *T = nullptr;
