@@ -542,6 +542,7 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   if (!mixed(ctx)) AL(ctx->rad, (size_t)C * B);
   AL(ctx->nH, C); AL(ctx->x5, 5 * (size_t)C); AL(ctx->T, C);
   AL(ctx->src_idx, C); AL(ctx->nsub, C); AL(ctx->status, 1);
+  AL(ctx->mask_in, C); AL(ctx->mask_norm, (size_t)C + 15); AL(ctx->mask_res, 1);
   ctx->stage_n = std::max<size_t>(4 * (size_t)B * C, 7 * (size_t)F);
   ctx->stage_n = std::max<size_t>(ctx->stage_n, 5 * (size_t)C);
   AL(ctx->stage, ctx->stage_n);
@@ -755,27 +756,32 @@ rt_status rt_set_active(rt_ctx* ctx, const uint8_t* active) {
   CK(cudaStreamSynchronize(ctx->stream), "rt_set_active");
   const int C = ctx->C, F = ctx->F, B = ctx->B;
   const int prev = ctx->cur_set;
-  std::vector<uint8_t> m;
-  bool all = true;
-  if (active) {
-    m.resize(C);
-    CK(cudaMemcpy(m.data(), active, (size_t)C, is_device_ptr(active) ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost),
-       "active mask");
-    for (int i = 0; i < C; ++i) {
-      m[i] = m[i] != 0;
-      all = all && m[i];
-    }
-  }
-  if (all) {
+  if (!active) {
     use_set(ctx, -1);
     return RT_OK;
   }
-  // a mask seen recently keeps its lists and its step graph
-  uint64_t h = 1469598103934665603ull;   // FNV-1a
-  for (uint8_t v : m) h = (h ^ v) * 1099511628211ull;
+  // compared on the device with the masks seen recently, which keep their
+  // lists and step graphs; on the legacy stream, as the copy, so that a device
+  // mask is read after the work that wrote it
+  static_assert(KnownMasks::kMax == rt_ctx::kMaxActSets, "one bit per kept set");
+  const size_t padded = ((size_t)C + 15) / 16 * 16;
+  KnownMasks known{};
+  for (int j = 0; j < rt_ctx::kMaxActSets; ++j) known.m[j] = ctx->sets[j].valid ? ctx->sets[j].mask : nullptr;
+  unsigned res = 0;
+  CK(cudaMemcpy(ctx->mask_in, active, (size_t)C, is_device_ptr(active) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice),
+     "active mask");
+  CK(cudaMemsetAsync(ctx->mask_res, 0, sizeof(unsigned), cudaStreamLegacy), "active mask");
+  k_match_mask<<<nblk((long long)padded / 16), kThreads, 0, cudaStreamLegacy>>>(C, ctx->mask_in, ctx->mask_norm, known,
+                                                                                 ctx->mask_res);
+  if ((st = launched(ctx, "active mask"))) return st;
+  CK(cudaMemcpy(&res, ctx->mask_res, sizeof(unsigned), cudaMemcpyDeviceToHost), "active mask");
+  if (!(res >> rt_ctx::kMaxActSets & 1u)) {
+    use_set(ctx, -1);
+    return RT_OK;
+  }
   int k = -1;
   for (int j = 0; j < rt_ctx::kMaxActSets && k < 0; ++j)
-    if (ctx->sets[j].valid && ctx->sets[j].hash == h && ctx->sets[j].mask == m) k = j;
+    if (ctx->sets[j].valid && !(res >> j & 1u)) k = j;
   if (k < 0) {
     // a free slot, else the least recently used one
     for (int j = 0; j < rt_ctx::kMaxActSets && k < 0; ++j)
@@ -787,6 +793,8 @@ rt_status rt_set_active(rt_ctx* ctx, const uint8_t* active) {
     }
     rt_ctx::ActSet& a = ctx->sets[k];
     free_set(a);
+    std::vector<uint8_t> m(padded);
+    CK(cudaMemcpy(m.data(), ctx->mask_norm, padded, cudaMemcpyDeviceToHost), "active mask");
     std::vector<int2> lr(F);
     if (F > 0) CK(cudaMemcpy(lr.data(), ctx->lr, (size_t)F * sizeof(int2), cudaMemcpyDeviceToHost), "active mask");
     std::vector<int32_t> ac, tc, af, gb;
@@ -837,7 +845,7 @@ rt_status rt_set_active(rt_ctx* ctx, const uint8_t* active) {
         (st = up(tc.data(), tc.size() * 4, (void**)&a.touched_cells)) ||
         (st = up(af.data(), af.size() * 4, (void**)&a.act_faces)) ||
         (st = up(gb.data(), gb.size() * 4, (void**)&a.grad_blocks)) ||
-        (st = up(tf.data(), tf.size(), (void**)&a.touched))) {
+        (st = up(tf.data(), tf.size(), (void**)&a.touched)) || (st = up(m.data(), m.size(), (void**)&a.mask))) {
       free_set(a);
       use_set(ctx, -1);
       return st;
@@ -847,8 +855,6 @@ rt_status rt_set_active(rt_ctx* ctx, const uint8_t* active) {
     a.n_act_faces = (int)af.size();
     a.n_grad_blocks = (int)gb.size();
     a.grad_cap_list = cap_list;
-    a.hash = h;
-    a.mask.swap(m);
     a.valid = true;
   }
   use_set(ctx, k);

@@ -81,8 +81,8 @@ struct rt_ctx {
   // through a few masks): their masks, device lists and step graphs
   struct ActSet {
     bool valid = false;
-    uint64_t hash = 0, used = 0;
-    std::vector<uint8_t> mask;
+    uint64_t used = 0;
+    uint8_t* mask = nullptr;   // device: 0 / 1 per cell, padded with ones to 16
     int32_t *act_cells = nullptr, *touched_cells = nullptr, *act_faces = nullptr, *grad_blocks = nullptr;
     uint8_t* touched = nullptr;
     int n_act = 0, n_touched = 0, n_act_faces = 0, n_grad_blocks = 0;
@@ -91,6 +91,8 @@ struct rt_ctx {
     GraphSlot graph;
   };
   static constexpr int kMaxActSets = 8;
+  uint8_t *mask_in = nullptr, *mask_norm = nullptr;   // a new mask, as given and normalised
+  unsigned* mask_res = nullptr;
   ActSet sets[kMaxActSets];
   int cur_set = -1;                    // -1: every cell active
   GraphSlot all_graph;                 // the step graph with every cell active
