@@ -102,11 +102,22 @@ void free_active(rt_ctx* ctx) {
   use_set(ctx, -1);
 }
 
+void adj_free(rt_ctx* ctx) {
+  for (void* p : ctx->adj.allocs) cudaFree(p);
+  ctx->adj = rt_ctx::Adj();
+}
+
+// Everything that belongs to the mesh: the buffers of its size (the source
+// rates and the reverse mode's among them) and the sources.
 void free_all(rt_ctx* ctx) {
   ctx->gen++;
   free_active(ctx);
+  adj_free(ctx);
   for (void* p : ctx->allocs) cudaFree(p);
   ctx->allocs.clear();
+  ctx->src_rate = nullptr;
+  ctx->src_cap = 0;
+  ctx->src_cells.clear();
   ctx->mesh_ready = false;
 }
 
@@ -1131,11 +1142,6 @@ template <class T> rt_status aalloc(rt_ctx* ctx, T** p, size_t n, const char* wh
   return RT_OK;
 }
 
-void adj_free(rt_ctx* ctx) {
-  for (void* p : ctx->adj.allocs) cudaFree(p);
-  ctx->adj = rt_ctx::Adj();
-}
-
 // The chemistry tape: room for `want` records (at least `need`, should
 // `want` not fit in device memory), keeping the first `keep`.
 rt_status tape_grow(rt_ctx* ctx, long long want, long long need, long long keep) {
@@ -1470,7 +1476,6 @@ void rt_destroy(rt_ctx* ctx) {
   cudaStreamSynchronize(ctx->stream);
   if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
-  adj_free(ctx);
   free_all(ctx);
   delete ctx;
 }
