@@ -6,6 +6,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/rt.h"
@@ -57,6 +58,26 @@ template <class T> rt_status dalloc(rt_ctx* ctx, T** p, size_t n, const char* wh
   ctx->allocs.push_back(q);
   *p = (T*)q;
   return RT_OK;
+}
+
+// Several device buffers in one allocation, each on a 256-byte boundary.
+struct Arena {
+  size_t bytes = 256;   // never empty
+  std::vector<std::pair<void**, size_t>> at;
+  void add_bytes(void** p, size_t n) {
+    at.push_back({p, bytes});
+    bytes += (std::max<size_t>(n, 1) + 255) / 256 * 256;
+  }
+  template <class T> void add(T** p, size_t n) { add_bytes((void**)p, n * sizeof(T)); }
+  void place(void* base) {
+    for (auto& a : at) *a.first = (char*)base + a.second;
+  }
+};
+
+// Before an error return with copies from the caller's memory under way.
+rt_status wait_fail(rt_ctx* ctx, rt_status st) {
+  cudaStreamSynchronize(ctx->stream);
+  return st;
 }
 
 void drop_graph(rt_ctx::GraphSlot& g) {
@@ -116,6 +137,7 @@ void free_all(rt_ctx* ctx) {
   for (void* p : ctx->allocs) cudaFree(p);
   ctx->allocs.clear();
   ctx->src_rate = nullptr;
+  ctx->src_cell = nullptr;
   ctx->src_cap = 0;
   ctx->src_cells.clear();
   ctx->mesh_ready = false;
@@ -486,133 +508,95 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   const int C = (int)cells->n, F = (int)faces->n, B = ctx->B;
   ctx->C = C;
   ctx->F = F;
-  // host copies for validation and the CSR build (these are the only host
-  // passes over the mesh)
-  std::vector<int32_t> L(F), Rr(F);
-  std::vector<double> V(C);
-  const bool dev_l = F > 0 && is_device_ptr(faces->left);
-  if (F > 0) {
-    CK(cudaMemcpy(L.data(), faces->left, F * 4, dev_l ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost), "mesh");
-    CK(cudaMemcpy(Rr.data(), faces->right, F * 4,
-                  is_device_ptr(faces->right) ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost), "mesh");
-  }
-  CK(cudaMemcpy(V.data(), cells->volume, (size_t)C * 8,
-                is_device_ptr(cells->volume) ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost), "mesh");
-  std::vector<int32_t> off(C + 1, 0);
-  for (int f = 0; f < F; ++f) {
-    if (L[f] < 0 || L[f] >= C || Rr[f] < 0 || Rr[f] >= C || L[f] == Rr[f])
-      return fail(ctx, RT_BAD_MESH, "face %d joins cells %d and %d (C = %d)", f, L[f], Rr[f], C);
-    off[L[f] + 1]++;
-    off[Rr[f] + 1]++;
-  }
-  double minV = INFINITY;
-  for (int i = 0; i < C; ++i) {
-    if (!(V[i] > 0) || !std::isfinite(V[i])) return fail(ctx, RT_BAD_MESH, "cell %d has volume %g", i, V[i]);
-    minV = std::min(minV, V[i]);
-  }
-  int maxdeg = 0;
-  for (int i = 0; i < C; ++i) {
-    maxdeg = std::max(maxdeg, off[i + 1]);
-    off[i + 1] += off[i];
-  }
-  for (int i = 0; i < C; ++i) {
-    if (off[i + 1] == off[i]) return fail(ctx, RT_BAD_MESH, "cell %d has no faces", i);
-  }
-  std::vector<int32_t> csr(2 * (size_t)F), nbr(2 * (size_t)F);
-  {
-    std::vector<int32_t> fill(off.begin(), off.end() - 1);
-    for (int f = 0; f < F; ++f) {     // ascending face index within each cell
-      nbr[fill[L[f]]] = Rr[f];
-      csr[fill[L[f]]++] = f << 1;
-      nbr[fill[Rr[f]]] = L[f];
-      csr[fill[Rr[f]]++] = (f << 1) | 1;
-    }
-  }
-  ctx->max_deg = maxdeg;
-  ctx->min_dx_cm = std::cbrt(minV) * ctx->cfg.unit_length_cm;
-  // staged gradients (FP32 sweep): shared memory for the largest block's
-  // half-edge records; a mesh whose blocks need more than kGradSmemMax keeps
-  // the unstaged kernel
-  ctx->grad_cap = 0;
-  if (mixed(ctx)) {
-    int cap = 0;
-    for (int c0 = 0; c0 < C; c0 += kGradCells) cap = std::max(cap, off[std::min(c0 + kGradCells, C)] - off[c0]);
-    const size_t smem = 2 * (size_t)cap * sizeof(float4);
-    if (smem <= kGradSmemMax) {
-      CK(allow_smem((const void*)k_grad_staged<kGradNB>), "staged gradients");
-      ctx->grad_cap = cap;
-    }
-  }
-
-  rt_status st;
-#define AL(p, n) if ((st = dalloc(ctx, &(p), (n), #p))) return st
-  AL(ctx->vol, C); AL(ctx->cx, C); AL(ctx->cy, C); AL(ctx->cz, C);
-  AL(ctx->off, C + 1); AL(ctx->csr, 2 * (size_t)F); AL(ctx->nbr, 2 * (size_t)F); AL(ctx->lr, F);
-  AL(ctx->nA64, F); AL(ctx->rL64, F); AL(ctx->rR64, F); AL(ctx->w64, F); AL(ctx->minv64, 6 * (size_t)C);
-  if (ctx->cfg.time_order == 2) AL(ctx->rad0, (size_t)C * B);
-  if (!mixed(ctx)) AL(ctx->rad, (size_t)C * B);
-  AL(ctx->nH, C); AL(ctx->x5, 5 * (size_t)C); AL(ctx->T, C);
-  AL(ctx->src_idx, C); AL(ctx->nsub, C); AL(ctx->status, 1);
-  AL(ctx->mask_in, C); AL(ctx->mask_norm, (size_t)C + 15); AL(ctx->mask_res, 1);
-  ctx->stage_n = std::max<size_t>(4 * (size_t)B * C, 7 * (size_t)F);
-  ctx->stage_n = std::max<size_t>(ctx->stage_n, 5 * (size_t)C);
-  AL(ctx->stage, ctx->stage_n);
   const bool mx = mixed(ctx);
-  const size_t rs = mx ? 4 : 8;
-  {
-    void* p;
-    const size_t gbytes = mx ? (size_t)C * 4 * pad_bins(B) * sizeof(float4) : (size_t)C * B * 12 * sizeof(double);
-    cudaError_t e = cudaMalloc(&p, std::max<size_t>(gbytes, 1));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "G");
-    ctx->allocs.push_back(p); ctx->G = p;
-    e = cudaMalloc(&p, std::max<size_t>((size_t)F * B * 4 * rs, 1));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "flux");
-    ctx->allocs.push_back(p); ctx->flux = p;
-    for (void** h : {&ctx->hw, &ctx->hx}) {
-      e = cudaMalloc(&p, std::max<size_t>(2 * (size_t)F * 4 * rs, 1));
-      if (e != cudaSuccess) return cuda_fail(ctx, e, "half-edges");
-      ctx->allocs.push_back(p); *h = p;
-    }
-    e = cudaMalloc(&p, std::max<size_t>((size_t)C * rs, 1));
-    if (e != cudaSuccess) return cuda_fail(ctx, e, "half-edges");
-    ctx->allocs.push_back(p); ctx->xmax = p;
-  }
-  AL(ctx->work_cell, C); AL(ctx->work_ctl, 4); AL(ctx->ivol, C);
+  const size_t rs = mx ? 4 : 8, c = C, f = F;
+  // one allocation for every buffer of the mesh's size
+  Arena ar;
+  MeshCheck* chk = nullptr;
+  ar.add(&chk, 1);
+  ar.add(&ctx->vol, c); ar.add(&ctx->cx, c); ar.add(&ctx->cy, c); ar.add(&ctx->cz, c);
+  ar.add(&ctx->off, c + 1); ar.add(&ctx->csr, 2 * f); ar.add(&ctx->nbr, 2 * f); ar.add(&ctx->lr, f);
+  ar.add(&ctx->nA64, f); ar.add(&ctx->rL64, f); ar.add(&ctx->rR64, f); ar.add(&ctx->w64, f);
+  ar.add(&ctx->minv64, 6 * c);
+  if (ctx->cfg.time_order == 2) ar.add(&ctx->rad0, c * B);
+  ar.add(&ctx->nH, c); ar.add(&ctx->x5, 5 * c); ar.add(&ctx->T, c);
+  ar.add(&ctx->src_idx, c); ar.add(&ctx->nsub, c); ar.add(&ctx->status, 1);
+  ar.add(&ctx->mask_in, c); ar.add(&ctx->mask_norm, c + 15); ar.add(&ctx->mask_res, 1);
+  ctx->stage_n = std::max<size_t>(std::max<size_t>(4 * (size_t)B * c, 7 * f), 5 * c);
+  ar.add(&ctx->stage, ctx->stage_n);
+  ar.add_bytes(&ctx->G, mx ? c * 4 * pad_bins(B) * sizeof(float4) : c * B * 12 * sizeof(double));
+  ar.add_bytes(&ctx->flux, f * B * 4 * rs);
+  ar.add_bytes(&ctx->hw, 2 * f * 4 * rs); ar.add_bytes(&ctx->hx, 2 * f * 4 * rs); ar.add_bytes(&ctx->xmax, c * rs);
+  ar.add(&ctx->work_cell, c); ar.add(&ctx->work_ctl, 4); ar.add(&ctx->ivol, c);
   if (mx) {
-    AL(ctx->fa32, F); AL(ctx->fb32, F);
-    AL(ctx->work_f1, C);
-    AL(ctx->shadow, (size_t)C * B);
-    AL(ctx->radN, (size_t)C * B);
+    ar.add(&ctx->fa32, f); ar.add(&ctx->fb32, f); ar.add(&ctx->work_f1, c);
+    ar.add(&ctx->shadow, c * B); ar.add(&ctx->radN, c * B);
   } else {
-    AL(ctx->work_f1d, C);
-    AL(ctx->hx32, 2 * (size_t)F);
+    ar.add(&ctx->rad, c * B); ar.add(&ctx->work_f1d, c); ar.add(&ctx->hx32, 2 * f);
   }
-#undef AL
-  if ((st = copy_in(ctx, ctx->vol, cells->volume, (size_t)C * 8))) return st;
-  if ((st = copy_in(ctx, ctx->cx, cells->cx, (size_t)C * 8))) return st;
-  if ((st = copy_in(ctx, ctx->cy, cells->cy, (size_t)C * 8))) return st;
-  if ((st = copy_in(ctx, ctx->cz, cells->cz, (size_t)C * 8))) return st;
-  CK(cudaMemcpyAsync(ctx->off, off.data(), (C + 1) * 4, cudaMemcpyHostToDevice, ctx->stream), "off");
-  CK(cudaMemcpyAsync(ctx->csr, csr.data(), 2 * (size_t)F * 4, cudaMemcpyHostToDevice, ctx->stream), "csr");
-  CK(cudaMemcpyAsync(ctx->nbr, nbr.data(), 2 * (size_t)F * 4, cudaMemcpyHostToDevice, ctx->stream), "nbr");
   {
-    std::vector<int2> lr(F);
-    for (int f = 0; f < F; ++f) lr[f] = make_int2(L[f], Rr[f]);
-    CK(cudaMemcpyAsync(ctx->lr, lr.data(), (size_t)F * 8, cudaMemcpyHostToDevice, ctx->stream), "lr");
-    CK(cudaStreamSynchronize(ctx->stream), "mesh upload");
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, ar.bytes);
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "mesh buffers");
+    ctx->allocs.push_back(p);
+    ar.place(p);
   }
+  rt_status st;
+  // device arrays may come from work on the legacy stream
+  CK(cudaStreamSynchronize(cudaStreamLegacy), "mesh");
+  // copies from the caller, all complete before this function returns
+  auto in = [&](void* dst, const void* src, size_t bytes) -> rt_status {
+    if (bytes == 0) return RT_OK;
+    CK(cudaMemcpyAsync(dst, src, bytes, is_device_ptr(src) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice,
+                       ctx->stream), "copy in");
+    return RT_OK;
+  };
+  // checks, degrees and face lists; both ids pass through the neighbour array,
+  // the degrees through the attempt counts, the fill marks through the worklist
+  int32_t *deg = ctx->nsub, *next = ctx->work_cell, *sums = ctx->src_idx;
+  if ((st = in(ctx->nbr, faces->left, f * 4)) || (st = in(ctx->nbr + f, faces->right, f * 4)) ||
+      (st = in(ctx->vol, cells->volume, c * 8)))
+    return wait_fail(ctx, st);
+  k_mesh_init<<<nblk(C), kThreads, 0, ctx->stream>>>(chk, ctx->x5, ctx->T, deg, C);
+  if (F > 0)
+    k_mesh_faces<<<nblk(F), kThreads, 0, ctx->stream>>>(F, C, ctx->nbr, ctx->nbr + f, ctx->lr, deg, chk);
+  k_mesh_cells<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->vol, deg, chk);
+  const int nbs = (C + kScan - 1) / kScan;
+  k_scan_blocks<<<nbs, kScan, 0, ctx->stream>>>(C, deg, ctx->off, sums);
+  k_scan_sums<<<1, kScan, 0, ctx->stream>>>(nbs, sums);
+  k_scan_add<<<nblk(C + 1LL), kThreads, 0, ctx->stream>>>(C, 2 * F, sums, ctx->off, next);
+  MeshCheck h{};
+  if ((st = launched(ctx, "mesh check"))) return wait_fail(ctx, st);
+  CK(cudaMemcpyAsync(&h, chk, sizeof h, cudaMemcpyDeviceToHost, ctx->stream), "mesh check");
+  CK(cudaStreamSynchronize(ctx->stream), "mesh check");
+  if (h.bad_face != kNoIndex) {
+    int2 b{};
+    CK(cudaMemcpy(&b, ctx->lr + h.bad_face, sizeof b, cudaMemcpyDeviceToHost), "mesh check");
+    return fail(ctx, RT_BAD_MESH, "face %d joins cells %d and %d (C = %d)", h.bad_face, b.x, b.y, C);
+  }
+  if (h.bad_volume != kNoIndex) {
+    double v = 0.0;
+    CK(cudaMemcpy(&v, ctx->vol + h.bad_volume, sizeof v, cudaMemcpyDeviceToHost), "mesh check");
+    return fail(ctx, RT_BAD_MESH, "cell %d has volume %g", h.bad_volume, v);
+  }
+  if (h.no_faces != kNoIndex) return fail(ctx, RT_BAD_MESH, "cell %d has no faces", h.no_faces);
+  double minV = 0.0;
+  std::memcpy(&minV, &h.min_volume, sizeof minV);
+  ctx->max_deg = h.max_deg;
+  ctx->min_dx_cm = std::cbrt(minV) * ctx->cfg.unit_length_cm;
+  k_mesh_fill<<<nblk(F), kThreads, 0, ctx->stream>>>(F, ctx->lr, ctx->off, next, ctx->csr);
+  k_mesh_sort<<<nblk(C), kThreads, 0, ctx->stream>>>(C, kGradCells, ctx->off, ctx->csr, ctx->lr, ctx->nbr, chk);
+  if ((st = launched(ctx, "face lists")) || (st = in(ctx->cx, cells->cx, c * 8)) || (st = in(ctx->cy, cells->cy, c * 8)) ||
+      (st = in(ctx->cz, cells->cz, c * 8)))
+    return wait_fail(ctx, st);
   // face arrays through the staging buffer: area, n, x_f
   double* sA = ctx->stage;
   double *snx = sA + F, *sny = sA + 2 * (size_t)F, *snz = sA + 3 * (size_t)F;
   double *sfx = sA + 4 * (size_t)F, *sfy = sA + 5 * (size_t)F, *sfz = sA + 6 * (size_t)F;
   if (F > 0) {
-    if ((st = copy_in(ctx, sA, faces->area, (size_t)F * 8))) return st;
-    if ((st = copy_in(ctx, snx, faces->nx, (size_t)F * 8))) return st;
-    if ((st = copy_in(ctx, sny, faces->ny, (size_t)F * 8))) return st;
-    if ((st = copy_in(ctx, snz, faces->nz, (size_t)F * 8))) return st;
-    if ((st = copy_in(ctx, sfx, faces->fx, (size_t)F * 8))) return st;
-    if ((st = copy_in(ctx, sfy, faces->fy, (size_t)F * 8))) return st;
-    if ((st = copy_in(ctx, sfz, faces->fz, (size_t)F * 8))) return st;
+    const double* src[] = {faces->area, faces->nx, faces->ny, faces->nz, faces->fx, faces->fy, faces->fz};
+    for (int k = 0; k < 7; ++k)
+      if ((st = in(sA + k * f, src[k], f * 8))) return wait_fail(ctx, st);
     k_pack_nA<<<nblk(F), kThreads, 0, ctx->stream>>>(F, snx, sny, snz, sA, ctx->nA64);
     k_geometry_faces<<<nblk(F), kThreads, 0, ctx->stream>>>(F, ctx->cfg.box, ctx->lr, ctx->cx, ctx->cy, ctx->cz,
                                                             sfx, sfy, sfz, sA, ctx->rL64, ctx->rR64, ctx->w64);
@@ -641,12 +625,21 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
     else
       k_cell_xmax<double><<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->off, (const d4*)ctx->hx, (double*)ctx->xmax);
   }
-  if ((st = launched(ctx, "geometry kernels"))) return st;
+  if ((st = launched(ctx, "geometry kernels"))) return wait_fail(ctx, st);
   int h_status = 0;
   CK(cudaMemcpyAsync(&h_status, ctx->status, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "status");
+  CK(cudaMemcpyAsync(&h, chk, sizeof h, cudaMemcpyDeviceToHost, ctx->stream), "status");
   CK(cudaStreamSynchronize(ctx->stream), "geometry");
   if (h_status & kStSingular) return fail(ctx, RT_BAD_MESH, "singular least-squares matrix (degenerate cell)");
-  // default state: no radiation, neutral gas at 1e4 K, no sources
+  // staged gradients (FP32 sweep): shared memory for the largest block's
+  // half-edge records; a mesh whose blocks need more than kGradSmemMax keeps
+  // the unstaged kernel
+  ctx->grad_cap = 0;
+  if (mx && 2 * (size_t)h.cap * sizeof(float4) <= kGradSmemMax) {
+    CK(allow_smem((const void*)k_grad_staged<kGradNB>), "staged gradients");
+    ctx->grad_cap = h.cap;
+  }
+  // default state: no radiation, neutral gas at 1e4 K (k_mesh_init), no sources
   if (mx) {
     CK(cudaMemsetAsync(ctx->radN, 0, (size_t)C * B * 8, ctx->stream), "state");
     CK(cudaMemsetAsync(ctx->shadow, 0, (size_t)C * B * sizeof(float4), ctx->stream), "state");
@@ -656,14 +649,6 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   CK(cudaMemsetAsync(ctx->nH, 0, (size_t)C * 8, ctx->stream), "state");
   CK(cudaMemsetAsync(ctx->nsub, 0, (size_t)C * 4, ctx->stream), "state");
   CK(cudaMemsetAsync(ctx->src_idx, 0xff, (size_t)C * 4, ctx->stream), "state");
-  {
-    std::vector<double> x(5 * (size_t)C, 0.0), T(C, 1e4);
-    std::fill(x.begin(), x.begin() + C, 1.0);
-    std::fill(x.begin() + 2 * (size_t)C, x.begin() + 3 * (size_t)C, 1.0);
-    CK(cudaMemcpyAsync(ctx->x5, x.data(), x.size() * 8, cudaMemcpyHostToDevice, ctx->stream), "state");
-    CK(cudaMemcpyAsync(ctx->T, T.data(), T.size() * 8, cudaMemcpyHostToDevice, ctx->stream), "state");
-    CK(cudaStreamSynchronize(ctx->stream), "state");
-  }
   ctx->n_src_cells = 0;
   ctx->mesh_ready = true;
   return RT_OK;
@@ -712,30 +697,37 @@ rt_status rt_set_sources(rt_ctx* ctx, int64_t n, const int64_t* cell, const doub
        "sources");
   }
   // bin rates per cell, summed in source order
-  std::vector<int32_t> idx(ctx->C, -1);
+  std::unordered_map<int64_t, int> index;
+  std::vector<int32_t> where;
   std::vector<double> rate;
-  int m = 0;
   for (int64_t k = 0; k < n; ++k) {
     if (hc[k] < 0 || hc[k] >= ctx->C) return fail(ctx, RT_INVALID_ARG, "source %lld in cell %lld out of range",
                                                   (long long)k, (long long)hc[k]);
-    int32_t& s = idx[hc[k]];
-    if (s < 0) {
-      s = m++;
-      rate.resize((size_t)m * B, 0.0);
+    const auto it = index.try_emplace(hc[k], (int)where.size());
+    if (it.second) {
+      where.push_back((int32_t)hc[k]);
+      rate.resize(where.size() * B, 0.0);
     }
-    for (int b = 0; b < B; ++b) rate[(size_t)s * B + b] += hq[(size_t)k * B + b];
+    for (int b = 0; b < B; ++b) rate[(size_t)it.first->second * B + b] += hq[(size_t)k * B + b];
   }
+  const int m = (int)where.size();
   if (m > ctx->src_cap) {
     double* p = nullptr;
-    if ((st = dalloc(ctx, &p, (size_t)m * B, "source rates"))) return st;
+    int32_t* w = nullptr;
+    if ((st = dalloc(ctx, &p, (size_t)m * B, "source rates")) || (st = dalloc(ctx, &w, (size_t)m, "source cells")))
+      return st;
     ctx->src_rate = p;
+    ctx->src_cell = w;
     ctx->src_cap = m;
   }
-  CK(cudaMemcpyAsync(ctx->src_idx, idx.data(), (size_t)ctx->C * 4, cudaMemcpyHostToDevice, ctx->stream),
-     "sources");
-  if (m > 0)
+  CK(cudaMemsetAsync(ctx->src_idx, 0xff, (size_t)ctx->C * 4, ctx->stream), "sources");
+  if (m > 0) {
     CK(cudaMemcpyAsync(ctx->src_rate, rate.data(), (size_t)m * B * 8, cudaMemcpyHostToDevice, ctx->stream),
        "sources");
+    CK(cudaMemcpyAsync(ctx->src_cell, where.data(), (size_t)m * 4, cudaMemcpyHostToDevice, ctx->stream), "sources");
+    k_mark_sources<<<nblk(m), kThreads, 0, ctx->stream>>>(m, ctx->src_cell, ctx->src_idx);
+    if ((st = launched(ctx, "sources"))) return st;
+  }
   CK(cudaStreamSynchronize(ctx->stream), "sources");
   ctx->gen++;   // the source pointer and count are launch arguments
   ctx->n_src_cells = m;

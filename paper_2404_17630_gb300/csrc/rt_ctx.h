@@ -40,6 +40,7 @@ struct rt_ctx {
   double *nH = nullptr, *x5 = nullptr, *T = nullptr;
   int32_t* src_idx = nullptr;
   double* src_rate = nullptr;
+  int32_t* src_cell = nullptr;   // the cell of each index
   int n_src_cells = 0, src_cap = 0;
   int32_t* nsub = nullptr;
   d4* rad0 = nullptr;          // state at the start of a Heun transport step (time_order 2)
