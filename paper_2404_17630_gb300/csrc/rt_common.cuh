@@ -172,7 +172,7 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
 // g <- g + (t - g^2) h with the remainder t - g^2 from one fused multiply-add
 // (Markstein, as div_nr) and h = 1 / (2 sqrt(t)) kept at the seed's 22 bits:
 // the seed's error 2^-22 becomes 2^-43 and then 2^-65, below half a unit in
-// the last place.  Six FP64 operations; the seed is the FP32 reciprocal
+// the last place.  Five FP64 operations; the seed is the FP32 reciprocal
 // square root of t's leading 24 bits scaled to [1, 4), its exponent set on
 // the integer pipe.  t = 0, the ends of the exponent range, negative t,
 // infinity and NaN take sqrt().
@@ -186,7 +186,7 @@ __device__ __forceinline__ double sqrt_nr(double t) {
   const double y = __hiloint2double((int)((((r >> 23) + 896u - (unsigned)half) << 20) | ((r & 0x7FFFFFu) >> 3)),
                                     (int)(r << 29));
   double g = t * y;
-  const double h = 0.5 * y;
+  const double h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));   // y / 2
   g = fma(fma(-g, g, t), h, g);
   return fma(fma(-g, g, t), h, g);
 }

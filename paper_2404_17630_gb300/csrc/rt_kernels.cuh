@@ -951,8 +951,10 @@ __global__ void __launch_bounds__(kGradCells* kMaxBins)
 
 // FP64: linear extrapolation of the cell state to the face centre, summed onto
 // the state by fused multiply-adds, clamped to N >= 0 and |F| <= c N (tested on
-// squares on the integer pipe; the square root only where it clamps).
-__device__ __forceinline__ void face_state(const d4& p, const double* __restrict__ Gp, const d4& x, double v[4]) {
+// squares on the integer pipe; the square root only where it clamps).  Also the
+// squares N2 = N^2 and fl2 = |F|^2 that the closure needs.
+__device__ __forceinline__ void face_state(const d4& p, const double* __restrict__ Gp, const d4& x, double v[4],
+                                           double& N2, double& fl2) {
   // the 12 gradient words of one (cell, bin) as three aligned 4-vectors
   const d4* G4 = reinterpret_cast<const d4*>(Gp);
   const d4 a = G4[0], b = G4[1], c = G4[2];
@@ -961,10 +963,12 @@ __device__ __forceinline__ void face_state(const d4& p, const double* __restrict
   for (int q = 0; q < 4; ++q)
     v[q] = fma(Gc[3 * q], x.x, fma(Gc[3 * q + 1], x.y, fma(Gc[3 * q + 2], x.z, comp<double>(p, q))));
   if (lt_zero(v[0])) v[0] = 0.0;
-  const double fl2 = v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
-  if (gt_nonneg(fl2, v[0] * v[0])) {
+  N2 = v[0] * v[0];
+  fl2 = v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
+  if (gt_nonneg(fl2, N2)) {
     const double s = v[0] / sqrt(fl2);
     v[1] *= s; v[2] *= s; v[3] *= s;
+    fl2 = N2;
   }
 }
 
@@ -1012,24 +1016,23 @@ __device__ __forceinline__ void m1_normal(const float v[4], float n0, float n1, 
 // (2 - r = 3 f^2 / (2 + r) takes the division by |F|^2 away): one square
 // root and one quotient per face state instead of three quotients and a root,
 // no case for F = 0, and no divisor that leaves the range of a fast quotient
-// where N is small.  The kernel is bound by the FP64 unit: 1.67 -> 1.06 ms per
-// launch at 250,047 cells, 234 -> 152 us at 262,144 cells with one bin.
-// Here: the two coefficients of N D n = a n / 3 + k F, and F . n.  s >= N
+// where N is small.  The kernel is bound by the FP64 unit: 1.67 -> 0.96 ms per
+// launch at 250,047 cells, 234 -> 138 us at 262,144 cells with one bin (1.06 and
+// 0.152 with the squares formed twice).
+// Here: the two coefficients of 3 N D n = a n + 9 k F, and F . n.  s >= N
 // (f <= 1, also where the squares are rounded or leave the normal range).
-__device__ __forceinline__ void m1_coef(const double v[4], double n0, double n1, double n2, double& a, double& k,
-                                        double& un) {
+__device__ __forceinline__ void m1_coef(const double v[4], double N2, double fl2, double n0, double n1, double n2,
+                                        double& a, double& k, double& un) {
   un = v[1] * n0 + v[2] * n1 + v[3] * n2;
-  const double fl2 = v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
   a = v[0];
   k = 0.0;
   // the tests on the integer pipe (v[0] >= 0 after the face-state clamp)
   if (gt_nonneg(v[0], 0.0) && gt_nonneg(fl2, 0.0)) {
-    const double N2 = v[0] * v[0];
     double t = fma(-3.0, fl2, 4.0 * N2);
     t = __double_as_longlong(N2) > __double_as_longlong(t) ? N2 : t;
     const double s = sqrt_nr(t);
     a = s - v[0];
-    k = div_nr(3.0 * un, fma(2.0, v[0], s));
+    k = div_nr(un, fma(2.0, v[0], s));
   }
 }
 
@@ -1086,18 +1089,18 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 6 : 1) k_flux(Geo<R> g, 
   if constexpr (sizeof(R) == 8) {
     const int2 c = __ldg(g.lr + f);
     const d4 nA = g.nA[f];
-    double vL[4], vR[4], aL, aR, kL, kR, uL, uR;
+    double vL[4], vR[4], N2L, N2R, f2L, f2R, aL, aR, kL, kR, uL, uR;
     const size_t sL = (size_t)c.x * B + b, sR = (size_t)c.y * B + b;
-    face_state(rad[sL], G + sL * 12, g.rL[f], vL);
-    face_state(rad[sR], G + sR * 12, g.rR[f], vR);
-    m1_coef(vL, nA.x, nA.y, nA.z, aL, kL, uL);
-    m1_coef(vR, nA.x, nA.y, nA.z, aR, kR, uR);
-    const double hA = 0.5 * nA.w, a3 = (aL + aR) * (1.0 / 3.0);
+    face_state(rad[sL], G + sL * 12, g.rL[f], vL, N2L, f2L);
+    face_state(rad[sR], G + sR * 12, g.rR[f], vR, N2R, f2R);
+    m1_coef(vL, N2L, f2L, nA.x, nA.y, nA.z, aL, kL, uL);
+    m1_coef(vR, N2R, f2R, nA.x, nA.y, nA.z, aR, kR, uR);
+    const double hA = 0.5 * nA.w, h3 = 1.5 * nA.w, a9 = (aL + aR) * (1.0 / 9.0);
     d4 o;
     o.x = hA * ((uL + uR) - (vR[0] - vL[0]));
-    o.y = hA * (fma(kR, vR[1], fma(kL, vL[1], a3 * nA.x)) - (vR[1] - vL[1]));
-    o.z = hA * (fma(kR, vR[2], fma(kL, vL[2], a3 * nA.y)) - (vR[2] - vL[2]));
-    o.w = hA * (fma(kR, vR[3], fma(kL, vL[3], a3 * nA.z)) - (vR[3] - vL[3]));
+    o.y = fma(h3, fma(kR, vR[1], fma(kL, vL[1], a9 * nA.x)), hA * (vL[1] - vR[1]));
+    o.z = fma(h3, fma(kR, vR[2], fma(kL, vL[2], a9 * nA.y)), hA * (vL[2] - vR[2]));
+    o.w = fma(h3, fma(kR, vR[3], fma(kL, vL[3], a9 * nA.z)), hA * (vL[3] - vR[3]));
     flux[t] = o;
   }
 }
