@@ -289,14 +289,14 @@ struct RateSlopes {
 
 __device__ RateSlopes rate_slopes(const TFns& t, const Rates& r) {
   RateSlopes d;
-  const double uH = exp(0.407 * (kLnAH - t.lnT)), uHe2 = exp(0.407 * (kLnAHe2 - t.lnT));
+  const double uH = kU407H * t.u407, uHe2 = kU407He2 * t.u407;
   d.aHII = -r.aHII * (1.5 - 2.242 * 0.407 * div_nr(uH, 1.0 + uH)) * t.iT;
   d.aHeIII = -r.aHeIII * (1.5 - 2.242 * 0.407 * div_nr(uHe2, 1.0 + uHe2)) * t.iT;
   // HeII: radiative 1.26e-14 lam^0.75 and dielectronic
   // 1.9e-3 T^-1.5 exp(-470000/T) (1 + 0.3 exp(-94000/T))
   const double iT2 = t.iT * t.iT;
-  const double rad = 1.26e-14 * exp(0.750 * (kLnLHe - t.lnT));
-  const double g = 1.9e-3 * div_nr(t.iT, t.sT) * t.e470;
+  const double rs = t.iT * t.sT, rad = (1.26e-14 * kLam075He) * (rs * sqrt_nr(rs));
+  const double g = 1.9e-3 * t.T15 * t.e470;
   d.aHeII = -0.75 * rad * t.iT +
             g * ((470000.0 * iT2 - 1.5 * t.iT) * (1.0 + 0.3 * t.e94) + 0.3 * t.e94 * 94000.0 * iT2);
   const double ts = -0.5 * (1.0 - t.tf) * t.iT;
@@ -330,7 +330,7 @@ __device__ CoolCoef cooling_coef(const TFns& t) {
   const double rH = 8.70e-27 * sT * t3, drH = rH * (0.5 * iT + lt3);
   const double rHe = 1.55e-26 * exp(0.3647 * t.lnT), drHe = rHe * 0.3647 * iT;
   const double rHe2 = 3.48e-26 * sT * t3, drHe2 = rHe2 * (0.5 * iT + lt3);
-  const double g = 1.24e-13 * div_nr(iT, sT) * t.e470;
+  const double g = 1.24e-13 * t.T15 * t.e470;
   const double di = g * (1.0 + 0.3 * t.e94);
   const double ddi = g * ((470000.0 * iT2 - 1.5 * iT) * (1.0 + 0.3 * t.e94) + 0.3 * t.e94 * 94000.0 * iT2);
   // bremsstrahlung with the Gaunt factor 1.1 + 0.34 exp(-(5.5 - log10 T)^2 / 3)

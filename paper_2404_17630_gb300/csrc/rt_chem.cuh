@@ -47,11 +47,11 @@ struct Rates {
 template <bool Fast> struct RateEval;
 
 // Functions of T shared by the FP64 rate fits and the cooling rate: every
-// power of T is exp(p (ln c - ln T)) from one logarithm, and the Boltzmann
-// factors that both use are formed once (relative error ~1e-15 against the
-// pow / exp of the definitions).
+// power of T from one logarithm or from sqrt(T) and 1 / T, the Boltzmann
+// factors that both use formed once (relative error ~1e-15 against the pow /
+// exp of the definitions).
 struct TFns {
-  double T, iT, sT, tf, lnT, e94, e470, e157, e285, e631;
+  double T, iT, sT, tf, lnT, e94, e470, e157, e285, e631, T15, u407;   // T^-3/2, T^-0.407
 };
 
 // natural logarithms of the fits' scale constants, and 1 / ln 10
@@ -65,49 +65,55 @@ constexpr double kInvLn10 = 0.43429448190325176;
 __device__ __forceinline__ TFns tfns(double T) {
   TFns t;
   t.T = T;
-  t.iT = div_nr(1.0, T);
-  t.sT = sqrt(T);
-  t.tf = div_nr(1.0, 1.0 + sqrt(T * 1e-5));
-  t.lnT = log(T);
+  t.iT = rcp_nr<2>(T);
+  t.sT = sqrt_nr(T);
+  t.tf = rcp_nr<2>(fma(t.sT, 0.0031622776601683794, 1.0));   // 1 / (1 + sqrt(T / 1e5))
+  t.lnT = log_series(T);
   t.e94 = exp(-94000.0 * t.iT);
-  t.e470 = exp(-470000.0 * t.iT);
+  const double e2 = t.e94 * t.e94;
+  t.e470 = e2 * e2 * t.e94;                                   // exp(-470000 / T)
   t.e157 = exp(-157809.1 * t.iT);
   t.e285 = exp(-285335.4 * t.iT);
   t.e631 = exp(-631515.0 * t.iT);
+  t.T15 = t.iT * t.iT * t.sT;
+  t.u407 = exp(-0.407 * t.lnT);
   return t;
 }
+
+// Constants of the fits' powers: 315614^1.5, 1263030^1.5 (lambda = 2 T_i / T of
+// HII and HeIII), (315614 / 2.740)^0.407, (1263030 / 2.740)^0.407, 570670^0.75.
+constexpr double kLam15H = 315614.0 * 561.7953363992976, kLam15He2 = 1263030.0 * 1123.8460748696862;
+constexpr double kU407H = 114.81327852071512, kU407He2 = 201.88817541951113, kLam075He = 20762.93678880667;
 
 template <> struct RateEval<false> {
   __device__ static Rates eval(const TFns& t) {
     Rates r;
     // Hui & Gnedin case B, lambda = 2 T_i / T: a lambda^1.5 / (1 + (lambda / 2.74)^0.407)^2.242
-    const double lH = 315614.0 * t.iT, lHe2 = 1263030.0 * t.iT;
-    const double uH = exp(0.407 * (kLnAH - t.lnT)), uHe2 = exp(0.407 * (kLnAHe2 - t.lnT));
-    r.aHII = 2.753e-14 * (lH * sqrt(lH)) * exp(-2.242 * log(1.0 + uH));
-    r.aHeIII = 2.0 * 2.753e-14 * (lHe2 * sqrt(lHe2)) * exp(-2.242 * log(1.0 + uHe2));
-    const double die = 1.9e-3 * div_nr(t.iT, t.sT) * t.e470 * (1.0 + 0.3 * t.e94);
-    r.aHeII = 1.26e-14 * exp(0.750 * (kLnLHe - t.lnT)) + die;
-    r.bHI = 5.85e-11 * t.sT * t.e157 * t.tf;
-    r.bHeI = 2.38e-11 * t.sT * t.e285 * t.tf;
-    r.bHeII = 5.68e-12 * t.sT * t.e631 * t.tf;
+    r.aHII = (2.753e-14 * kLam15H) * t.T15 * exp(-2.242 * log_series(fma(kU407H, t.u407, 1.0)));
+    r.aHeIII = (2.0 * 2.753e-14 * kLam15He2) * t.T15 * exp(-2.242 * log_series(fma(kU407He2, t.u407, 1.0)));
+    const double die = 1.9e-3 * t.T15 * t.e470 * fma(0.3, t.e94, 1.0);
+    const double rs = t.iT * t.sT;   // T^-1/2
+    r.aHeII = fma(1.26e-14 * kLam075He, rs * sqrt_nr(rs), die);
+    const double st = t.sT * t.tf;
+    r.bHI = 5.85e-11 * st * t.e157;
+    r.bHeI = 2.38e-11 * st * t.e285;
+    r.bHeII = 5.68e-12 * st * t.e631;
     return r;
   }
   __device__ static Rates eval(double T) { return eval(tfns(T)); }
+  // from the species' densities, grouped by species
   __device__ static double cooling(const TFns& t, double ne, double nHI, double nHII, double nHeI, double nHeII,
                                    double nHeIII) {
-    const double sT = t.sT, tf = t.tf;
-    const double ce = 7.50e-19 * exp(-118348.0 * t.iT) * tf * ne * nHI +
-                      5.54e-17 * exp(-0.397 * t.lnT) * exp(-473638.0 * t.iT) * tf * ne * nHeII;
-    const double ci = 1.27e-21 * sT * t.e157 * tf * ne * nHI + 9.38e-22 * sT * t.e285 * tf * ne * nHeI +
-                      4.95e-22 * sT * t.e631 * tf * ne * nHeII;
-    const double t3 = div_nr(exp(-0.2 * (t.lnT - kLn1e3)), 1.0 + exp(0.7 * (t.lnT - kLn1e6)));
-    const double rc = 8.70e-27 * sT * t3 * ne * nHII + 1.55e-26 * exp(0.3647 * t.lnT) * ne * nHeII +
-                      3.48e-26 * sT * t3 * ne * nHeIII +
-                      1.24e-13 * div_nr(t.iT, sT) * t.e470 * (1.0 + 0.3 * t.e94) * ne * nHeII;
-    const double lg = t.lnT * kInvLn10;
-    const double gff = 1.1 + 0.34 * exp(div_nr(-(5.5 - lg) * (5.5 - lg), 3.0));
-    const double br = 1.42e-27 * gff * sT * (nHII + nHeII + 4.0 * nHeIII) * ne;
-    return ce + ci + rc + br;
+    const double st = t.sT * t.tf;
+    const double kHI = fma(7.50e-19 * t.tf, exp(-118348.0 * t.iT), 1.27e-21 * st * t.e157);
+    const double kHeI = 9.38e-22 * st * t.e285;
+    const double t3 = t.sT * div_nr(exp(-0.2 * (t.lnT - kLn1e3)), 1.0 + exp(0.7 * (t.lnT - kLn1e6)));
+    const double d = 5.5 - t.lnT * kInvLn10;
+    const double br = 1.42e-27 * fma(0.34, exp(d * d * (-1.0 / 3.0)), 1.1) * t.sT;
+    const double kHeII = fma(5.54e-17 * t.tf, exp(fma(-473638.0, t.iT, -0.397 * t.lnT)), 4.95e-22 * st * t.e631) +
+                         fma(1.55e-26, exp(0.3647 * t.lnT), 1.24e-13 * t.T15 * t.e470 * fma(0.3, t.e94, 1.0));
+    return ne * (kHI * nHI + kHeI * nHeI + (kHeII + br) * nHeII + fma(8.70e-27, t3, br) * nHII +
+                 fma(3.48e-26, t3, 4.0 * br) * nHeIII);
   }
 };
 
@@ -195,90 +201,125 @@ __device__ __forceinline__ double rel_change(double a, double b, double fl) {
   return div_nr(fabs(b - a), m);
 }
 
+// The largest of n relative changes |b - a| / max(|a|, floor).  Each is formed
+// in FP32 first (relative error below 1e-6: differences in FP64, cut to FP32,
+// one quotient); a leader that is 4e-6 ahead of all others is the largest, and
+// only its quotient is formed in FP64.  Otherwise (and with values outside
+// the FP32 range or not finite) all of them are.
+template <int n>
+__device__ __forceinline__ double largest_change(const double a[n], const double b[n], const double fl[n], int use) {
+  float m1 = 0.0f, m2 = 0.0f;
+  double num = 0.0, den = 1.0;
+  bool ok = true;
+#pragma unroll
+  for (int q = 0; q < n; ++q) {
+    if (q >= use) continue;
+    const double d = fabs(b[q] - a[q]);
+    const double m = __double_as_longlong(fabs(a[q])) > __double_as_longlong(fl[q]) ? fabs(a[q]) : fl[q];
+    const float df = d2f_int(d), mf = d2f_int(m);
+    const float r = __fdividef(df, mf);
+    ok = ok && mf > 1e-36f && r < 1e30f && (df > 0.0f || __double_as_longlong(d) == 0);
+    if (r > m1) { num = d; den = m; }
+    m2 = fmaxf(m2, fminf(m1, r));
+    m1 = fmaxf(m1, r);
+  }
+  if (ok && m1 > 1e-30f && m1 - m2 > 4e-6f * m1) return div_nr(num, den);
+  double f = 0.0;
+#pragma unroll
+  for (int q = 0; q < n; ++q)
+    if (q < use) f = fmax(f, rel_change(a[q], b[q], fl[q]));
+  return f;
+}
+
 // One semi-implicit photochemistry attempt over dt from s into t; returns the
 // largest relative change f of the substep rule.  Steps: radiation level
 // over the step (implicit in N, absorbers at the start); photoionisation
 // rates from it; backward Euler for H, then for He with the updated n_e;
 // photons removed = photoionisations credited (absorbers at the end), F scaled
-// alike; thermal energy explicit.
+// alike; thermal energy explicit.  Arranged for the FP64 unit, which bounds it:
+// one reciprocal per denominator, the photons' factor 1 - (c dt sum sigma n') /
+// (1 + c dt sum sigma n) instead of a quotient by N, thirteen exponentials, one
+// quotient for the measure.
 __device__ double photochem_attempt(const ChemParams& P, double nH, double dt, const CellState& s, CellState& t) {
   const int B = P.B;
-  const double c = P.c_red;
+  const double cdt = P.c_red * dt;
   const double nHe = P.y_he * nH;
   const bool recomb = P.flags & 1, coll = P.flags & 2, cool = P.flags & 4, heat = P.flags & 8;
   const TFns tfn = tfns(s.T);
   const Rates r = RateEval<false>::eval(tfn);
 
-  double ns0 = nH * s.xHI, ns1 = nHe * s.yI, ns2 = nHe * s.yII;
-  double Nbar[kMaxBins];
-  double G0 = 0, G1 = 0, G2 = 0;
+  const double ns[3] = {nH * s.xHI, nHe * s.yI, nHe * s.yII};
+  double inv[kMaxBins], Nbar[kMaxBins];
+  double G[3] = {0.0, 0.0, 0.0};
 #pragma unroll
   for (int b = 0; b < kMaxBins; ++b) {
     if (b < B) {
-      double kap = P.sigma[b][0] * ns0 + P.sigma[b][1] * ns1 + P.sigma[b][2] * ns2;
-      Nbar[b] = div_nr(s.N[b], 1.0 + c * dt * kap);
-      G0 += c * P.sigma[b][0] * Nbar[b];
-      G1 += c * P.sigma[b][1] * Nbar[b];
-      G2 += c * P.sigma[b][2] * Nbar[b];
+      double kap = 0.0;
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (P.smask & (1 << (3 * b + q))) kap = fma(P.sigma[b][q], ns[q], kap);
+      inv[b] = rcp_nr<2>(fma(cdt, kap, 1.0));
+      Nbar[b] = cdt * (s.N[b] * inv[b]);
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (P.smask & (1 << (3 * b + q))) G[q] = fma(P.sigma[b][q], Nbar[b], G[q]);
     }
   }
-  double ne0 = nH * s.xHII + nHe * (s.yII + 2.0 * s.yIII);
-  double aH = dt * (G0 + (coll ? r.bHI * ne0 : 0.0));
-  double bH = recomb ? dt * r.aHII * ne0 : 0.0;
-  double den = 1.0 + aH + bH;
-  t.xHI = div_nr(s.xHI * (1.0 + bH) + bH * s.xHII, den);
-  t.xHII = div_nr(s.xHII * (1.0 + aH) + aH * s.xHI, den);
-  double ne1 = nH * t.xHII + nHe * (s.yII + 2.0 * s.yIII);
-  double A = dt * (G1 + (coll ? r.bHeI * ne1 : 0.0));
-  double Bb = recomb ? dt * r.aHeII * ne1 : 0.0;
-  double Cc = dt * (G2 + (coll ? r.bHeII * ne1 : 0.0));
-  double D = recomb ? dt * r.aHeIII * ne1 : 0.0;
-  double opA = 1.0 + A, opD = 1.0 + D;
-  t.yII = div_nr(s.yII + div_nr(A * s.yI, opA) + div_nr(D * s.yIII, opD), 1.0 + div_nr(Bb, opA) + div_nr(Cc, opD));
-  t.yI = div_nr(s.yI + Bb * t.yII, opA);
-  t.yIII = div_nr(s.yIII + Cc * t.yII, opD);
+  const double ne_he = nHe * fma(2.0, s.yIII, s.yII);
+  const double ne0 = fma(nH, s.xHII, ne_he);
+  const double aH = coll ? fma(dt, r.bHI * ne0, G[0]) : G[0];
+  const double bH = recomb ? dt * (r.aHII * ne0) : 0.0;
+  const double iden = rcp_nr<2>(1.0 + aH + bH), xs = s.xHI + s.xHII;
+  t.xHI = fma(bH, xs, s.xHI) * iden;
+  t.xHII = fma(aH, xs, s.xHII) * iden;
+  const double ne1 = fma(nH, t.xHII, ne_he);
+  const double A = coll ? fma(dt, r.bHeI * ne1, G[1]) : G[1];
+  const double Cc = coll ? fma(dt, r.bHeII * ne1, G[2]) : G[2];
+  const double Bb = recomb ? dt * (r.aHeII * ne1) : 0.0, D = recomb ? dt * (r.aHeIII * ne1) : 0.0;
+  const double iA = rcp_nr<2>(1.0 + A), iD = rcp_nr<2>(1.0 + D);
+  t.yII = div_nr(fma(D * iD, s.yIII, fma(A * iA, s.yI, s.yII)), fma(Cc, iD, fma(Bb, iA, 1.0)));
+  t.yI = fma(Bb, t.yII, s.yI) * iA;
+  t.yIII = fma(Cc, t.yII, s.yIII) * iD;
 
-  double m0 = nH * t.xHI, m1 = nHe * t.yI, m2 = nHe * t.yII;
+  const double m[3] = {nH * t.xHI, nHe * t.yI, nHe * t.yII};
   double heat_e = 0.0;
 #pragma unroll
   for (int b = 0; b < kMaxBins; ++b) {
     if (b < B) {
-      double i0 = c * dt * Nbar[b] * P.sigma[b][0] * m0;
-      double i1 = c * dt * Nbar[b] * P.sigma[b][1] * m1;
-      double i2 = c * dt * Nbar[b] * P.sigma[b][2] * m2;
-      heat_e += P.eps[b][0] * i0 + P.eps[b][1] * i1 + P.eps[b][2] * i2;
-      double N1 = s.N[b] - ((i0 + i1) + i2);
-      if (N1 < 0) N1 = 0;
-      double sc = s.N[b] > 0 ? div_nr(N1, s.N[b]) : 0.0;
-      t.N[b] = N1;
+      double sum = 0.0, ea = 0.0;
+#pragma unroll
+      for (int q = 0; q < 3; ++q)
+        if (P.smask & (1 << (3 * b + q))) {
+          const double sn = P.sigma[b][q] * m[q];
+          sum += sn;
+          if (heat && (P.emask & (1 << (3 * b + q)))) ea = fma(P.eps[b][q], sn, ea);
+        }
+      if (heat) heat_e = fma(Nbar[b], ea, heat_e);
+      double sc = fma(-(cdt * sum), inv[b], 1.0);
+      sc = __double_as_longlong(sc) > 0 ? sc : 0.0;
+      t.N[b] = s.N[b] * sc;
+      if (!(__double_as_longlong(s.N[b]) > 0)) sc = 0.0;
       t.f[b][0] = s.f[b][0] * sc;
       t.f[b][1] = s.f[b][1] * sc;
       t.f[b][2] = s.f[b][2] * sc;
     }
   }
-  double f = 0.0;
+  double e0 = 0.0, e1 = 0.0;
+  t.T = s.T;
   if (P.mode == 2) {
-    double ntot0 = nH * (1.0 + P.y_he) + ne0;
-    double e0 = 1.5 * kBoltzmann * ntot0 * s.T;
-    double lam = cool ? RateEval<false>::cooling(tfn, ne0, nH * s.xHI, nH * s.xHII, nHe * s.yI, nHe * s.yII,
-                                                nHe * s.yIII)
-                      : 0.0;
-    double e1 = e0 + (heat ? heat_e : 0.0) - dt * lam;
-    double ne2 = nH * t.xHII + nHe * (t.yII + 2.0 * t.yIII);
-    double ntot1 = nH * (1.0 + P.y_he) + ne2;
-    t.T = div_nr(e1, 1.5 * kBoltzmann * ntot1);
-    f = rel_change(e0, e1, 0.0);
-  } else {
-    t.T = s.T;
+    const double nn = nH * (1.0 + P.y_he);
+    e0 = 1.5 * kBoltzmann * (nn + ne0) * s.T;
+    const double lam = cool ? RateEval<false>::cooling(tfn, ne0, ns[0], nH * s.xHII, ns[1], ns[2], nHe * s.yIII) : 0.0;
+    e1 = fma(-dt, lam, e0 + heat_e);
+    const double ne2 = fma(nH, t.xHII, nHe * fma(2.0, t.yIII, t.yII));
+    t.T = div_nr(e1, 1.5 * kBoltzmann * (nn + ne2));
   }
-  f = fmax(f, rel_change(s.xHI, t.xHI, P.x_floor));
-  f = fmax(f, rel_change(s.xHII, t.xHII, P.x_floor));
-  if (P.y_he > 0) {
-    f = fmax(f, rel_change(s.yI, t.yI, P.x_floor));
-    f = fmax(f, rel_change(s.yII, t.yII, P.x_floor));
-    f = fmax(f, rel_change(s.yIII, t.yIII, P.x_floor));
-  }
-  return f;
+  // (the energy's base has no floor; without thermal energy its change is 0)
+  const double xf = P.x_floor;
+  const double a[6] = {P.mode == 2 ? e0 : 1.0, s.xHI, s.xHII, s.yI, s.yII, s.yIII};
+  const double b[6] = {P.mode == 2 ? e1 : 1.0, t.xHI, t.xHII, t.yI, t.yII, t.yIII};
+  const double fl[6] = {0.0, xf, xf, xf, xf, xf};
+  return largest_change<6>(a, b, fl, P.y_he > 0 ? 6 : 3);
 }
 
 // FP64 reciprocal: FP32 hardware seed (~22 bits) refined by one Newton step

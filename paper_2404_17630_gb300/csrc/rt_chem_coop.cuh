@@ -27,41 +27,6 @@ constexpr unsigned kFull = 0xffffffffu;
 template <class T> __device__ __forceinline__ T from_lane(T v, int src) { return __shfl_sync(kFull, v, src, kGroup); }
 template <class T> __device__ __forceinline__ T xor_lane(T v, int m) { return __shfl_xor_sync(kFull, v, m, kGroup); }
 
-// 1 / x by a seed and one (relative error 2^-44, as rcp64) or two (below one
-// unit in the last place) Newton-Raphson steps.
-template <int kSteps> __device__ __forceinline__ double rcp_nr(double x) {
-  double y;
-  if (!rcp_seed(x, y)) return 1.0 / x;
-#pragma unroll
-  for (int k = 0; k < kSteps; ++k) y = fma(y, fma(-x, y, 1.0), y);
-  return y;
-}
-
-// ln x for normal x > 0: x = m 2^e with m in [sqrt(1/2), sqrt(2)), ln m = 2
-// artanh(s), s = (m - 1) / (m + 1), from the series of artanh: |s| <= 0.172,
-// the first term left out is 2e-17 of the sum.  22 FP64 instructions.  Other
-// x take log().
-__device__ __forceinline__ double log_series(double x) {
-  const int hi = __double2hiint(x);
-  if ((unsigned)(hi - 0x00100000) >= 0x7FE00000u) return log(x);
-  const int e = (hi - 0x3FE6A09E) >> 20;   // m >= sqrt(1/2)
-  const double m = __hiloint2double(hi - (e << 20), __double2loint(x));
-  const double s = div_nr(m - 1.0, m + 1.0), z = s * s;
-  double p = 1.0 / 21.0;
-  p = fma(p, z, 1.0 / 19.0);
-  p = fma(p, z, 1.0 / 17.0);
-  p = fma(p, z, 1.0 / 15.0);
-  p = fma(p, z, 1.0 / 13.0);
-  p = fma(p, z, 1.0 / 11.0);
-  p = fma(p, z, 1.0 / 9.0);
-  p = fma(p, z, 1.0 / 7.0);
-  p = fma(p, z, 1.0 / 5.0);
-  p = fma(p, z, 1.0 / 3.0);
-  const double s2 = 2.0 * s;
-  const double r = fma(s2 * z, p, s2);
-  return fma((double)e, 0.6931471805599453, fma((double)e, 2.3190468138462996e-17, r));
-}
-
 // What each lane evaluates: E = exp(p (q - ln T) + r / T), and its share of
 // the rates (kr) and of the cooling rate (kc) from V = F E P with the lane's
 // factor F (fsel: 0 none, 1 tf, 2 sqrt(T) tf, 3 sqrt(T), 4 T^-3/2) and
