@@ -597,14 +597,13 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
     const double* src[] = {faces->area, faces->nx, faces->ny, faces->nz, faces->fx, faces->fy, faces->fz};
     for (int k = 0; k < 7; ++k)
       if ((st = in(sA + k * f, src[k], f * 8))) return wait_fail(ctx, st);
-    k_pack_nA<<<nblk(F), kThreads, 0, ctx->stream>>>(F, snx, sny, snz, sA, ctx->nA64);
-    k_geometry_faces<<<nblk(F), kThreads, 0, ctx->stream>>>(F, ctx->cfg.box, ctx->lr, ctx->cx, ctx->cy, ctx->cz,
-                                                            sfx, sfy, sfz, sA, ctx->rL64, ctx->rR64, ctx->w64);
+    k_geometry_faces<<<nblk(F), kThreads, 0, ctx->stream>>>(F, make_box(ctx->cfg.box), ctx->lr, ctx->cx, ctx->cy,
+                                                            ctx->cz, snx, sny, snz, sfx, sfy, sfz, sA, ctx->nA64,
+                                                            ctx->rL64, ctx->rR64, ctx->w64);
   }
   CK(cudaMemsetAsync(ctx->status, 0, sizeof(int), ctx->stream), "status");
   CK(cudaMemsetAsync(ctx->work_ctl, 0, 4 * sizeof(int), ctx->stream), "worklist");
-  k_geometry_cells<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->cfg.box, ctx->off, ctx->csr, ctx->lr, ctx->cx,
-                                                          ctx->cy, ctx->cz, sA, ctx->minv64, ctx->status);
+  k_geometry_cells<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->off, ctx->csr, ctx->w64, ctx->minv64, ctx->status);
   if (mx && F > 0) {
     k_build_facerecs<<<nblk(F), kThreads, 0, ctx->stream>>>(F, ctx->lr, ctx->nA64, ctx->rL64, ctx->rR64, ctx->fa32,
                                                             ctx->fb32);

@@ -1,6 +1,7 @@
 // Shared device-side types and helpers of the M1 RT subcycle kernels.
 #pragma once
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 namespace m1rt {
@@ -82,10 +83,31 @@ template <class R> __device__ __forceinline__ R mk(double v) { return static_cas
 __device__ __forceinline__ double rint_away(double x) { return round(x); }
 __device__ __forceinline__ float rint_away(float x) { return roundf(x); }
 
-// Periodic minimum image of a coordinate difference, d - L round(d / L),
-// evaluated without contraction so that it rounds like the plain expression.
-__device__ __forceinline__ double min_image(double d, double L) {
-  return L > 0.0 ? __dsub_rn(d, __dmul_rn(L, round(__ddiv_rn(d, L)))) : d;
+// Periodic box of side L (0: not periodic) with the high words of 0.4999 L,
+// 0.5001 L and 1.4999 L.
+struct Box {
+  double L;
+  int h_in, h_out, h_two;
+};
+inline Box make_box(double L) {
+  auto hi = [](double v) {
+    long long b;
+    std::memcpy(&b, &v, sizeof b);
+    return (int)(b >> 32);
+  };
+  return Box{L, hi(0.4999 * L), hi(0.5001 * L), hi(1.4999 * L)};
+}
+
+// Periodic minimum image of a coordinate difference, d - L round(d / L): d
+// itself within 0.4999 L, d -+ L between 0.5001 L and 1.4999 L (told apart by
+// the high words on the integer pipe), elsewhere the expression itself,
+// evaluated without contraction so that it rounds like the plain one.
+__device__ __forceinline__ double min_image(double d, const Box& b) {
+  if (!(b.L > 0.0)) return d;
+  const int hi = __double2hiint(d), h = hi & 0x7FFFFFFF;
+  if (h < b.h_in) return d;
+  if (h > b.h_out && h < b.h_two) return __dsub_rn(d, hi < 0 ? -b.L : b.L);
+  return __dsub_rn(d, __dmul_rn(b.L, round(__ddiv_rn(d, b.L))));
 }
 
 // Precision conversions on the integer pipe.  GB300's FP64 pipe is its

@@ -10,7 +10,6 @@
 // keeps its cells' geometry in shared memory.
 #include <cstdint>
 #include <cstdio>
-#include <cstring>
 
 #include <cuda_runtime.h>
 
@@ -44,8 +43,7 @@ using namespace m1rt;
 
 struct NoallocArgs {
   int C, B;
-  double box;
-  int h_in, h_out, h_two;   // high words of 0.4999, 0.5001 and 1.4999 box (box > 0)
+  Box box;
   int limiter;
   double lim_eps2;
   const int32_t *off, *csr, *left, *right;
@@ -53,17 +51,6 @@ struct NoallocArgs {
   double* G;
   int* bad;
 };
-
-// Minimum image, d - L round(d / L): d itself within 0.4999 L, d -+ L between
-// 0.5001 L and 1.4999 L (told apart by the high words), the expression
-// elsewhere.
-__device__ __forceinline__ double mimg(double d, const NoallocArgs& a) {
-  if (!(a.box > 0.0)) return d;
-  const int hi = __double2hiint(d), h = hi & 0x7FFFFFFF;
-  if (h < a.h_in) return d;
-  if (h > a.h_out && h < a.h_two) return __dsub_rn(d, hi < 0 ? -a.box : a.box);
-  return __dsub_rn(d, __dmul_rn(a.box, round(__ddiv_rn(d, a.box))));
-}
 
 // Half-edge k of cell i: the weight w = A d / |d|^2 towards the neighbour j and
 // the face-centre offset x with |x|^2.
@@ -74,13 +61,13 @@ __device__ __forceinline__ HalfEdge half_edge(const NoallocArgs& a, int i, int k
   const int e = a.csr[k], f = e >> 1;
   const int j = (e & 1) ? a.left[f] : a.right[f];
   const double c0 = a.cx[i], c1 = a.cy[i], c2 = a.cz[i];
-  d[0] = mimg(a.cx[j] - c0, a);
-  d[1] = mimg(a.cy[j] - c1, a);
-  d[2] = mimg(a.cz[j] - c2, a);
+  d[0] = min_image(a.cx[j] - c0, a.box);
+  d[1] = min_image(a.cy[j] - c1, a.box);
+  d[2] = min_image(a.cz[j] - c2, a.box);
   const double s = div_nr(a.area[f], d[0] * d[0] + d[1] * d[1] + d[2] * d[2]);
   HalfEdge h;
   h.w = make_d4(s * d[0], s * d[1], s * d[2], id_bits(j, 0.0));
-  const double x0 = mimg(a.fx[f] - c0, a), x1 = mimg(a.fy[f] - c1, a), x2 = mimg(a.fz[f] - c2, a);
+  const double x0 = min_image(a.fx[f] - c0, a.box), x1 = min_image(a.fy[f] - c1, a.box), x2 = min_image(a.fz[f] - c2, a.box);
   h.x = make_d4(x0, x1, x2, x0 * x0 + x1 * x1 + x2 * x2);
   return h;
 }
@@ -241,12 +228,6 @@ __global__ void __launch_bounds__(kNaCells * 3) k_noalloc_grad(NoallocArgs a) {
   }
 }
 
-int high_word(double v) {
-  uint64_t b;
-  std::memcpy(&b, &v, sizeof b);
-  return (int)(b >> 32);
-}
-
 // Device memory of the current device `dev`, or managed memory.  Device memory
 // of another GPU is refused: the kernels run on `dev` and would otherwise read
 // another GPU's memory (a fault, or peer traffic where peer access is on).
@@ -302,8 +283,7 @@ rt_status rt_gradients_noalloc(const rt_cells* cells, const rt_faces* faces, con
     return set_err(RT_CUDA, "rt_gradients_noalloc: memset failed");
   }
   NoallocArgs a{};
-  a.C = Ci; a.B = n_bins; a.box = box;
-  a.h_in = high_word(0.4999 * box); a.h_out = high_word(0.5001 * box); a.h_two = high_word(1.4999 * box);
+  a.C = Ci; a.B = n_bins; a.box = make_box(box);
   a.limiter = limiter; a.lim_eps2 = lim_eps * lim_eps;
   a.off = cell_off; a.csr = cell_faces; a.left = faces->left; a.right = faces->right;
   a.cx = cells->cx; a.cy = cells->cy; a.cz = cells->cz; a.area = faces->area;
