@@ -552,8 +552,9 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
     return RT_OK;
   };
   // checks, degrees and face lists; both ids pass through the neighbour array,
-  // the degrees through the attempt counts, the fill marks through the worklist
-  int32_t *deg = ctx->nsub, *next = ctx->work_cell, *sums = ctx->src_idx;
+  // the degrees through the attempt counts, the fill marks through the
+  // worklist, the prefix sums' parts through the staging buffer
+  int32_t *deg = ctx->nsub, *next = ctx->work_cell, *sums = (int32_t*)ctx->stage;
   if ((st = in(ctx->nbr, faces->left, f * 4)) || (st = in(ctx->nbr + f, faces->right, f * 4)) ||
       (st = in(ctx->vol, cells->volume, c * 8)))
     return wait_fail(ctx, st);
@@ -795,67 +796,69 @@ rt_status rt_set_active(rt_ctx* ctx, const uint8_t* active) {
     }
     rt_ctx::ActSet& a = ctx->sets[k];
     free_set(a);
-    std::vector<uint8_t> m(padded);
-    CK(cudaMemcpy(m.data(), ctx->mask_norm, padded, cudaMemcpyDeviceToHost), "active mask");
-    std::vector<int2> lr(F);
-    if (F > 0) CK(cudaMemcpy(lr.data(), ctx->lr, (size_t)F * sizeof(int2), cudaMemcpyDeviceToHost), "active mask");
-    std::vector<int32_t> ac, tc, af, gb;
-    std::vector<uint8_t> tf(C, 0);
-    for (int i = 0; i < C; ++i)
-      if (m[i]) ac.push_back(i);
-    for (int f = 0; f < F; ++f)
-      if (m[lr[f].x] || m[lr[f].y]) {
-        af.push_back(f);
-        tf[lr[f].x] = tf[lr[f].y] = 1;
-      }
-    for (int i = 0; i < C; ++i)
-      if (tf[i]) tc.push_back(i);
-    for (int c0 = 0; c0 < C; c0 += kGradCells) {
-      bool any = false;
-      for (int i = c0; i < std::min(c0 + kGradCells, C) && !any; ++i) any = tf[i];
-      if (any) gb.push_back(c0 / kGradCells);
+    // flags and counts first, the lists once their lengths are known.  The
+    // flags of faces and blocks and the partial counts lie in the staging
+    // buffer (7 F doubles at least).
+    const int nblock = (C + kGradCells - 1) / kGradCells;
+    auto parts = [](int n) { return (n + kScan - 1) / kScan; };
+    uint8_t* face = (uint8_t*)ctx->stage;
+    uint8_t* block = face + ((size_t)F + 15) / 16 * 16;
+    int32_t* sums = (int32_t*)(block + ((size_t)nblock + 15) / 16 * 16);
+    int32_t *s_act = sums, *s_touched = s_act + parts(C) + 1, *s_face = s_touched + parts(C) + 1,
+            *s_block = s_face + parts(F) + 1;
+    int* cap = (int*)ctx->mask_res;
+    cudaStream_t q = cudaStreamLegacy;
+    uint8_t* touched = ctx->mask_in;   // its contents are in mask_norm
+    CK(cudaMemsetAsync(touched, 0, (size_t)C, q), "active lists");
+    CK(cudaMemsetAsync(cap, 0, sizeof(int), q), "active lists");
+    k_set_faces<<<nblk(F), kThreads, 0, q>>>(F, ctx->lr, ctx->mask_norm, face, touched);
+    k_set_blocks<<<nblk(nblock), kThreads, 0, q>>>(nblock, C, kGradCells, touched, block);
+    struct { int n; const uint8_t* flag; int32_t* sums; } job[] = {
+        {C, ctx->mask_norm, s_act}, {C, touched, s_touched}, {F, face, s_face}, {nblock, block, s_block}};
+    for (auto& j : job) {
+      k_flag_count<<<parts(j.n), kScan, 0, q>>>(j.n, j.flag, j.sums);
+      k_scan_sums<<<1, kScan, 0, q>>>(parts(j.n), j.sums);
     }
+    if ((st = launched(ctx, "active lists"))) return st;
+    int count[4] = {};
+    for (int i = 0; i < 4; ++i)
+      CK(cudaMemcpyAsync(count + i, job[i].sums + parts(job[i].n), sizeof(int), cudaMemcpyDeviceToHost, q), "active lists");
+    CK(cudaStreamSynchronize(q), "active lists");
+    Arena ar;
+    ar.add(&a.act_cells, count[0]); ar.add(&a.touched_cells, count[1]); ar.add(&a.act_faces, count[2]);
+    ar.add(&a.grad_blocks, count[3]); ar.add(&a.touched, C); ar.add(&a.mask, padded);
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, ar.bytes);
+    if (e != cudaSuccess) {
+      free_set(a);
+      use_set(ctx, -1);
+      return cuda_fail(ctx, e, "active lists");
+    }
+    a.allocs.push_back(p);
+    ar.place(p);
+    int32_t* list[] = {a.act_cells, a.touched_cells, a.act_faces, a.grad_blocks};
+    for (int i = 0; i < 4; ++i)
+      k_flag_list<<<parts(job[i].n), kScan, 0, q>>>(job[i].n, job[i].flag, job[i].sums, list[i]);
     // staged gradients over the touched list: the face records of the
     // largest block of kGradCells list entries must fit in shared memory
+    if (mixed(ctx) && ctx->grad_cap > 0 && count[1] > 0)
+      k_list_cap<<<nblk((count[1] + kGradCells - 1) / kGradCells), kThreads, 0, q>>>(count[1], kGradCells,
+                                                                                     a.touched_cells, ctx->off, cap);
     int cap_list = 0;
-    if (mixed(ctx) && ctx->grad_cap > 0) {
-      std::vector<int32_t> deg(C, 0);
-      for (int f = 0; f < F; ++f) {
-        deg[lr[f].x]++;
-        deg[lr[f].y]++;
-      }
-      for (size_t j0 = 0; j0 < tc.size(); j0 += kGradCells) {
-        int sum = 0;
-        for (size_t j = j0; j < std::min(j0 + kGradCells, tc.size()); ++j) sum += deg[tc[j]];
-        cap_list = std::max(cap_list, sum);
-      }
-      if (2 * (size_t)cap_list * sizeof(float4) > kGradSmemMax) cap_list = 0;
-    }
-    auto up = [&](const void* src, size_t bytes, void** dst) -> rt_status {
-      void* p = nullptr;
-      cudaError_t e = cudaMalloc(&p, std::max<size_t>(bytes, 16));
-      if (e != cudaSuccess) return cuda_fail(ctx, e, "active lists");
-      a.allocs.push_back(p);
-      if (bytes) {
-        e = cudaMemcpy(p, src, bytes, cudaMemcpyHostToDevice);
-        if (e != cudaSuccess) return cuda_fail(ctx, e, "active lists");
-      }
-      *dst = p;
-      return RT_OK;
-    };
-    if ((st = up(ac.data(), ac.size() * 4, (void**)&a.act_cells)) ||
-        (st = up(tc.data(), tc.size() * 4, (void**)&a.touched_cells)) ||
-        (st = up(af.data(), af.size() * 4, (void**)&a.act_faces)) ||
-        (st = up(gb.data(), gb.size() * 4, (void**)&a.grad_blocks)) ||
-        (st = up(tf.data(), tf.size(), (void**)&a.touched)) || (st = up(m.data(), m.size(), (void**)&a.mask))) {
+    if ((st = launched(ctx, "active lists"))) {
       free_set(a);
       use_set(ctx, -1);
       return st;
     }
-    a.n_act = (int)ac.size();
-    a.n_touched = (int)tc.size();
-    a.n_act_faces = (int)af.size();
-    a.n_grad_blocks = (int)gb.size();
+    CK(cudaMemcpyAsync(a.touched, touched, (size_t)C, cudaMemcpyDeviceToDevice, q), "active lists");
+    CK(cudaMemcpyAsync(a.mask, ctx->mask_norm, padded, cudaMemcpyDeviceToDevice, q), "active lists");
+    CK(cudaMemcpyAsync(&cap_list, cap, sizeof(int), cudaMemcpyDeviceToHost, q), "active lists");
+    CK(cudaStreamSynchronize(q), "active lists");
+    if (2 * (size_t)cap_list * sizeof(float4) > kGradSmemMax) cap_list = 0;
+    a.n_act = count[0];
+    a.n_touched = count[1];
+    a.n_act_faces = count[2];
+    a.n_grad_blocks = count[3];
     a.grad_cap_list = cap_list;
     a.valid = true;
   }
