@@ -31,7 +31,7 @@ namespace m1rt {
 // is N D n = ((s - N) / 3) n + k F, s = sqrt(4 N^2 - 3 |F|^2), k = 3 (F . n) /
 // (2 N + s) (m1_coef), smooth at F = 0; its two quotients share one reciprocal,
 // of (2 N + s) s.  The clamps (N >= 0, |F| <= N) as face_state.  Bound by the
-// FP64 unit: 794 -> 629 us per launch at 74,088 cells, three bins.
+// FP64 unit: 794 -> 552 us per launch at 74,088 cells, three bins.
 __device__ __forceinline__ d4 adj_side(const d4& p, const double* __restrict__ Gp, const d4& x, double n0, double n1,
                                        double n2, const double lP[3], double third, double lN, const double l0[3]) {
   const d4* G4 = reinterpret_cast<const d4*>(Gp);
@@ -44,8 +44,10 @@ __device__ __forceinline__ d4 adj_side(const d4& p, const double* __restrict__ G
   const double N = clampN ? 0.0 : e0, N2 = N * N, q2 = e1 * e1 + e2 * e2 + e3 * e3;
   const bool clampF = gt_nonneg(q2, N2);
   double F1 = e1, F2 = e2, F3 = e3, fl2 = q2;
+  double ifl = 0.0;
   if (clampF) {
-    const double r = N / sqrt(q2);
+    ifl = div_nr(1.0, sqrt_nr(q2));
+    const double r = N * ifl;
     F1 *= r; F2 *= r; F3 *= r;
     fl2 = N2;
   }
@@ -69,7 +71,6 @@ __device__ __forceinline__ d4 adj_side(const d4& p, const double* __restrict__ G
     lN += third;
   }
   if (clampF) {
-    const double ifl = div_nr(1.0, sqrt(q2));
     const double lvf = (lf1 * e1 + lf2 * e2 + lf3 * e3) * ifl, z = N * ifl, y = lvf * ifl;
     lN += lvf;
     lf1 = z * (lf1 - y * e1);

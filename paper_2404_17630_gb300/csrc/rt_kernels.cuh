@@ -646,13 +646,10 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
     const R4<R> hw = ld4<R>(g.hw + k);
     acc_face(hw, ld4<R>(rad + (size_t)bits_id(hw.w) * B + b));
   }
-  R gg[4], psi[4];
+  R psi[4];
   int lim_at[4] = {-1, -1, -1, -1}, lim_cell[4] = {-1, -1, -1, -1};
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    gg[q] = gr[q][0] * gr[q][0] + gr[q][1] * gr[q][1] + gr[q][2] * gr[q][2];
-    psi[q] = R(1);
-  }
+  for (int q = 0; q < 4; ++q) psi[q] = R(1);
   if (limiter) {
     // psi = min over faces of (max - phi_i) / (g.x) for g.x > 0 and
     // (min - phi_i) / (g.x) for g.x < 0.  Rounded division is monotone in
@@ -664,13 +661,11 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
     if constexpr (sizeof(R) == 4) {
       float eg[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) eg[q] = sqrtf(lim_eps2 * gg[q]);
+      for (int q = 0; q < 4; ++q)
+        eg[q] = sqrtf(lim_eps2 * (gr[q][0] * gr[q][0] + gr[q][1] * gr[q][1] + gr[q][2] * gr[q][2]));
       lim_extremes(g.hx, k0, k1, gr, eg, __ldg(g.xmax + i), dpos, dneg);
     } else {
-      R thr[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) thr[q] = lim_eps2 * gg[q];
-      lim_extremes(g.hx, g.hx32, k0, k1, gr, thr, __ldg(g.xmax + i), dpos, dneg, at);
+      lim_extremes(g.hx, g.hx32, k0, k1, gr, lim_eps2, __ldg(g.xmax + i), dpos, dneg, at);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
@@ -686,12 +681,12 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
       if constexpr (sizeof(R) == 8) {
         // dpos >= +0, dneg = -magnitude or +0, the factors >= +0: the
         // tests on the integer pipe
-        if (gt_nonneg(dpos[q], 0.0)) {
+        if (limits_pos(up, dpos[q])) {
           const R lim = div_nr(up, dpos[q]);
           if (kTape && gt_nonneg(psi[q], lim)) { lim_at[q] = at[2 * q]; lim_cell[q] = jmx[q]; }
           psi[q] = gt_nonneg(psi[q], lim) ? lim : psi[q];
         }
-        if (__double_as_longlong(dneg[q]) != 0) {
+        if (limits_neg(dn, dneg[q])) {
           const R lim = div_nr(dn, dneg[q]);
           // equal factors: the face that comes first
           if (kTape && (gt_nonneg(psi[q], lim) ||
@@ -1004,7 +999,7 @@ __device__ __forceinline__ void face_state(const d4& p, const double* __restrict
   N2 = v[0] * v[0];
   fl2 = v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
   if (gt_nonneg(fl2, N2)) {
-    const double s = v[0] / sqrt(fl2);
+    const double s = div_nr(v[0], sqrt_nr(fl2));
     v[1] *= s; v[2] *= s; v[3] *= s;
     fl2 = N2;
   }

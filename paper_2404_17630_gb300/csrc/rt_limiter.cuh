@@ -37,8 +37,9 @@ __device__ __forceinline__ bool lt_zero(double x) {
 
 // g scaled by a power of two so that its largest component lies in [1, 2),
 // cut to FP32 on the integer pipe (relative error below 2^-23; components
-// 2^-126 of the largest become zero).  false where that has no meaning: g = 0,
-// subnormal or not finite.
+// 2^-126 of the largest become zero).  false where the largest lies outside
+// 2^-400 .. 2^400 (g = 0 or not finite among them): the squares of the
+// regularisation test stay in the normal range only inside.
 __device__ __forceinline__ bool scaled_f32(const double g[3], float o[3]) {
   unsigned hi[3], top = 0;
 #pragma unroll
@@ -53,26 +54,30 @@ __device__ __forceinline__ bool scaled_f32(const double g[3], float o[3]) {
     const unsigned m = ((hi[d] & 0xFFFFFu) << 3) | ((unsigned)__double2loint(g[d]) >> 29);
     o[d] = __uint_as_float((hi[d] & 0x80000000u) | (e > 0 ? ((unsigned)e << 23) | m : 0u));
   }
-  return top != 0u && top != 0x7FF00000u;
+  return (top >> 20) - 623u < 800u;
 }
 
 // Limiter extremes of one (cell, bin) in FP64: dpos = max(0, max g.x_f) and
 // dneg = min(0, min g.x_f) over the faces k0..k1-1 that pass the
-// regularisation test, which compares squares (thr = eps^2 |g|^2, X the
-// largest x.w = |x_f|^2), and the extremes are kept as bit patterns (integer
-// compares; the FP64 pipe is the kernel's bound).  First a search in FP32 for
-// the face that attains each extreme: |g| scaled to below 2 per component,
-// the FP32 product g . x_f is within 6 2^-24 2 (|x| + |y| + |z|) <= 1.3e-6 |x_f|
-// of the exact one (both operands rounded, three roundings of the sum), so a
-// leader that is 2.6e-6 of the cell's largest |x_f| ahead of every other face
-// and of zero is the FP64 leader, and its FP64 product is the extreme: eight
-// FP64 products per (cell, bin) instead of four per face (with the matrix
-// folded into the weights: 0.85 -> 0.54 ms per launch at 250,047 cells).  Where a lead is
-// smaller (faces that tie by symmetry; a leader within the band of zero) every
-// face's product is formed in FP64.  A component without gradient has no
-// extremes.  at[2q], at[2q + 1]: the first face that attains dpos[q], dneg[q].
+// regularisation test (g.x_f)^2 > eps2 |g|^2 |x_f|^2 (X: the largest x.w =
+// |x_f|^2), kept as bit patterns (integer compares; the FP64 pipe is the
+// kernel's bound).  First a search in FP32 for the face that attains each
+// extreme: |g| scaled to below 2 per component, the FP32 product g . x_f is
+// within 6 2^-24 2 (|x| + |y| + |z|) <= 1.3e-6 |x_f| of the exact one (both
+// operands rounded, three roundings of the sum), so a leader that is 2.6e-6 of
+// the cell's largest |x_f| ahead of every other face and of zero is the FP64
+// leader, and its FP64 product is the extreme: eight FP64 products per (cell,
+// bin) instead of four per face (with the matrix folded into the weights:
+// 0.85 -> 0.52 ms per launch at 250,047 cells, 142 -> 82 us at 262,144 cells of six
+// faces and one bin).  A leader beyond the test's bound
+// for the largest |x_f|, by the same margin, also passes its own test, and
+// nothing more is to be tested: rounding is monotone.  Where a lead is smaller
+// (faces that tie by symmetry; a leader within the band of zero) every face's
+// product is formed in FP64 and, where an extreme does not clear the bound,
+// tested.  A component without gradient has no extremes.  at[2q], at[2q + 1]: the
+// first face that attains dpos[q], dneg[q].
 __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const float4* __restrict__ xf, int k0, int k1,
-                                             const double gr[4][3], const double thr[4], double X, double dpos[4],
+                                             const double gr[4][3], double eps2, double X, double dpos[4],
                                              double dneg[4], int at[8]) {
   float gf[4][3], m1[8], m2[8];
   bool flat[4], sure = true;
@@ -100,11 +105,16 @@ __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const fl
       }
     }
   }
-  const float lead = 2.6e-6f * sqrtf((float)X);
+  const float xm = sqrtf((float)X);
+  sure = sure && xm > 1e-18f && xm < 1e18f;
+  const float ex = 1.0001f * sqrtf((float)eps2) * xm, lead = 2.6e-6f * xm;
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < 4; ++q) {
+    const float clear = fmaf(ex, sqrtf(gf[q][0] * gf[q][0] + gf[q][1] * gf[q][1] + gf[q][2] * gf[q][2]), lead);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) sure = sure && (flat[q] || m1[2 * q + h] - m2[2 * q + h] > lead);
+    for (int h = 0; h < 2; ++h)
+      sure = sure && (flat[q] || (m1[2 * q + h] - m2[2 * q + h] > lead && m1[2 * q + h] > clear));
+  }
   long long bpos[4], bneg[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) bpos[q] = bneg[q] = 0;
@@ -117,6 +127,8 @@ __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const fl
       bneg[q] = max_bits_neg(0, gr[q][0] * c.x + gr[q][1] * c.y + gr[q][2] * c.z);
     }
   } else {
+    bool exact = true;
+    double thr[4];
 #pragma unroll 1
     for (int k = k0; k < k1; ++k) {
       const d4 x = ld4<double>(xs + k);
@@ -130,30 +142,30 @@ __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const fl
         bneg[q] = n;
       }
     }
-  }
-  bool exact = true;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const long long t = __double_as_longlong(thr[q] * X);
-    const double p = __longlong_as_double(bpos[q]), n = neg_from_bits(bneg[q]);
-    exact = exact && (bpos[q] == 0 || __double_as_longlong(p * p) > t) &&
-            (bneg[q] == 0 || __double_as_longlong(n * n) > t);
-  }
-  if (!exact) {
+    for (int q = 0; q < 4; ++q) {
+      thr[q] = eps2 * (gr[q][0] * gr[q][0] + gr[q][1] * gr[q][1] + gr[q][2] * gr[q][2]);
+      const long long t = __double_as_longlong(thr[q] * X);
+      const double p = __longlong_as_double(bpos[q]), n = neg_from_bits(bneg[q]);
+      exact = exact && (bpos[q] == 0 || __double_as_longlong(p * p) > t) &&
+              (bneg[q] == 0 || __double_as_longlong(n * n) > t);
+    }
+    if (!exact) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) bpos[q] = bneg[q] = 0;
+      for (int q = 0; q < 4; ++q) bpos[q] = bneg[q] = 0;
 #pragma unroll 1
-    for (int k = k0; k < k1; ++k) {
-      const d4 x = ld4<double>(xs + k);
+      for (int k = k0; k < k1; ++k) {
+        const d4 x = ld4<double>(xs + k);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const double dphi = gr[q][0] * x.x + gr[q][1] * x.y + gr[q][2] * x.z;
-        if (__double_as_longlong(dphi * dphi) > __double_as_longlong(thr[q] * x.w)) {
-          const long long p = max_bits_pos(bpos[q], dphi), n = max_bits_neg(bneg[q], dphi);
-          at[2 * q] = p != bpos[q] ? k : at[2 * q];
-          at[2 * q + 1] = n != bneg[q] ? k : at[2 * q + 1];
-          bpos[q] = p;
-          bneg[q] = n;
+        for (int q = 0; q < 4; ++q) {
+          const double dphi = gr[q][0] * x.x + gr[q][1] * x.y + gr[q][2] * x.z;
+          if (__double_as_longlong(dphi * dphi) > __double_as_longlong(thr[q] * x.w)) {
+            const long long p = max_bits_pos(bpos[q], dphi), n = max_bits_neg(bneg[q], dphi);
+            at[2 * q] = p != bpos[q] ? k : at[2 * q];
+            at[2 * q + 1] = n != bneg[q] ? k : at[2 * q + 1];
+            bpos[q] = p;
+            bneg[q] = n;
+          }
         }
       }
     }
@@ -164,5 +176,11 @@ __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const fl
     dneg[q] = neg_from_bits(bneg[q]);
   }
 }
+
+// The limiter factor from the extremes: min(1, up / dpos, dn / dneg) with up, dn
+// the largest and most negative difference to a neighbour.  The quotients are
+// formed only where they are below 1 (tested on the integer pipe).
+__device__ __forceinline__ bool limits_pos(double up, double dpos) { return gt_nonneg(dpos, up); }
+__device__ __forceinline__ bool limits_neg(double dn, double dneg) { return gt_nonneg(-dneg, -dn); }
 
 }  // namespace m1rt

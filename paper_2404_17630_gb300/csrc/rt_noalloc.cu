@@ -173,22 +173,25 @@ __global__ void __launch_bounds__(kNaCells * 3) k_noalloc_grad(NoallocArgs a) {
       dn[q] = max_bits_neg(dn[q], dphi);
     }
   }
-  double g[4][3], thr[4], psi[4];
+  double g[4][3], psi[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     g[q][0] = i00 * r[q][0] + i01 * r[q][1] + i02 * r[q][2];
     g[q][1] = i01 * r[q][0] + i11 * r[q][1] + i12 * r[q][2];
     g[q][2] = i02 * r[q][0] + i12 * r[q][1] + i22 * r[q][2];
-    thr[q] = a.lim_eps2 * (g[q][0] * g[q][0] + g[q][1] * g[q][1] + g[q][2] * g[q][2]);
     psi[q] = 1.0;
   }
   if (a.limiter) {
     double dpos[4], dneg[4];
     if (staged) {
       int at[8];
-      lim_extremes(sx, sf, k0 - kb, k1 - kb, g, thr, __longlong_as_double(X), dpos, dneg, at);
+      lim_extremes(sx, sf, k0 - kb, k1 - kb, g, a.lim_eps2, __longlong_as_double(X), dpos, dneg, at);
     } else {
       long long p[4] = {0, 0, 0, 0}, q4[4] = {0, 0, 0, 0};
+      double thr[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        thr[q] = a.lim_eps2 * (g[q][0] * g[q][0] + g[q][1] * g[q][1] + g[q][2] * g[q][2]);
       for (int k = k0; k < k1; ++k) {
         const d4 x = half_edge(a, i, k, d).x;
 #pragma unroll
@@ -210,11 +213,11 @@ __global__ void __launch_bounds__(kNaCells * 3) k_noalloc_grad(NoallocArgs a) {
     for (int q = 0; q < 4; ++q) {
       // the smallest quotient is the one by the largest g . x: rounded division
       // is monotone in the divisor
-      if (gt_nonneg(dpos[q], 0.0)) {
+      if (limits_pos(__longlong_as_double(up[q]), dpos[q])) {
         const double lim = div_nr(__longlong_as_double(up[q]), dpos[q]);
         psi[q] = gt_nonneg(psi[q], lim) ? lim : psi[q];
       }
-      if (__double_as_longlong(dneg[q]) != 0) {
+      if (limits_neg(neg_from_bits(dn[q]), dneg[q])) {
         const double lim = div_nr(neg_from_bits(dn[q]), dneg[q]);
         psi[q] = gt_nonneg(psi[q], lim) ? lim : psi[q];
       }
