@@ -29,9 +29,8 @@ namespace m1rt {
 // state (lN and lf, the parts that do not go through the closure) and of N D n
 // (lP, with third = lP . n / 3) to those of the extrapolated state.  The closure
 // is N D n = ((s - N) / 3) n + k F, s = sqrt(4 N^2 - 3 |F|^2), k = 3 (F . n) /
-// (2 N + s) (m1_coef), smooth at F = 0; its two quotients share one reciprocal,
-// of (2 N + s) s.  The clamps (N >= 0, |F| <= N) as face_state.  Bound by the
-// FP64 unit: 794 -> 552 us per launch at 74,088 cells, three bins.
+// (2 N + s) (m1_coef), smooth at F = 0.  The clamps (N >= 0, |F| <= N) as face_state.
+// Bound by the FP64 unit: 794 -> 552 us per launch at 74,088 cells, three bins.
 __device__ __forceinline__ d4 adj_side(const d4& p, const double* __restrict__ Gp, const d4& x, double n0, double n1,
                                        double n2, const double lP[3], double third, double lN, const double l0[3]) {
   const d4* G4 = reinterpret_cast<const d4*>(Gp);
@@ -56,7 +55,9 @@ __device__ __forceinline__ d4 adj_side(const d4& p, const double* __restrict__ G
     double t = fma(-3.0, fl2, 4.0 * N2);
     t = gt_nonneg(N2, t) ? N2 : t;
     const double s = sqrt_nr(t), d = fma(2.0, N, s);
-    const double r = rcp_nr<2>(d * s), id3 = 3.0 * (r * s), is = r * d;
+    // (one reciprocal of d s would leave the exponent range at densities that
+    // occur beyond a light front: N^2 < 1e-308)
+    const double id3 = 3.0 * rcp_nr<2>(d), is = rcp_nr<2>(s);
     const double un = F1 * n0 + F2 * n1 + F3 * n2;
     const double lPF = lP[0] * F1 + lP[1] * F2 + lP[2] * F3;
     const double k = un * id3, lun = lPF * id3;
