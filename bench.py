@@ -390,8 +390,8 @@ def e2e_measure(precision, mesh, cfg, state, steps, warmup, dev):
 # steady state), per cell for the FP64 sweep kernels.  The unit counts behind
 # the `alu` rooflines; re-measured after each change of these kernels.
 FP64_FLOP = {
-    "mixed": {"k_chem": (159.0, "attempt")},
-    "fp64": {"k_chem": (1238.0, "attempt"), "k_grad": (2762.4, "cell"), "k_flux": (5673.8, "cell"),
+    "mixed": {"k_chem": (139.0, "attempt")},
+    "fp64": {"k_chem": (887.0, "attempt"), "k_grad": (1484.1, "cell"), "k_flux": (3618.9, "cell"),
              "k_gather": (439.4, "cell")},
 }
 # FP64-pipe instructions (thread instructions on the FP64 pipe, ncu
@@ -400,9 +400,9 @@ FP64_FLOP = {
 # at a saturated FP64 pipe is below the DFMA-stream peak; the instruction
 # rate against the stream's (peak FLOP / 2 per DFMA) is the pipe's use.
 FP64_INST = {
-    "mixed": {"k_chem": (109.1, "attempt")},
-    "fp64": {"k_chem": (801.0, "attempt"), "k_grad": (1944.5, "cell"), "k_flux": (3803.6, "cell"),
-             "k_gather": (282.0, "cell")},
+    "mixed": {"k_chem": (92.1, "attempt")},
+    "fp64": {"k_chem": (553.2, "attempt"), "k_grad": (1106.0, "cell"), "k_flux": (2213.0, "cell"),
+             "k_gather": (282.4, "cell")},
 }
 # Fallback FP64 peak from unit counts and clock, used only when the
 # measurement (rt_fp64_peak) is not available: 152 SMs x 2 FP64 FMA lanes per

@@ -30,7 +30,7 @@ namespace m1rt {
 // (lP, with third = lP . n / 3) to those of the extrapolated state.  The closure
 // is N D n = ((s - N) / 3) n + k F, s = sqrt(4 N^2 - 3 |F|^2), k = 3 (F . n) /
 // (2 N + s) (m1_coef), smooth at F = 0.  The clamps (N >= 0, |F| <= N) as face_state.
-// Bound by the FP64 unit: 794 -> 552 us per launch at 74,088 cells, three bins.
+// Bound by the FP64 unit: 794 -> 561 us per launch at 74,088 cells, three bins.
 __device__ __forceinline__ d4 adj_side(const d4& p, const double* __restrict__ Gp, const d4& x, double n0, double n1,
                                        double n2, const double lP[3], double third, double lN, const double l0[3]) {
   const d4* G4 = reinterpret_cast<const d4*>(Gp);

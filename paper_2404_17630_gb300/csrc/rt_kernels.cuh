@@ -1,5 +1,6 @@
 // Kernels of the M1 RT subcycle.
 //
+//   k_mesh_*, k_scan_*  once per mesh: checks and per-cell face lists
 //   k_geometry_*   once per mesh (Sec. 2.3.2: the least-squares matrix depends
 //                  only on geometry and is inverted once)
 //   k_grad<R>      least-squares gradients + slope limiter, one thread per
@@ -8,10 +9,10 @@
 //                  thread per (face, bin)  (Sec. 2.3.3, 4.1.3)
 //   k_gather<R>    per (cell, bin): deterministic CSR gather of the stored
 //                  face fluxes, FP64 update (Sec. 4.1.3)
-//   k_chem         per cell: source injection and thermochemistry (Eq. E,
-//                  Sec. 2.3.1, 4.1.1), FP64 sweep
-//   k_chem_first,  the same in two passes for the mixed precision
-//   k_chem_rest    (first attempt of every cell, then the rejected cells)
+//   k_chem_first,  source injection and thermochemistry (Eq. E, Sec. 2.3.1,
+//   k_chem_rest    4.1.1) in two passes, mixed precision: the first attempt of
+//                  every cell, then the rejected cells
+//   k_chem64_*     the same in FP64
 //
 // R is the precision of the transport sweep (double, or float in the mixed
 // mode of Sec. 6.2); the master state, the gather sums, the volume divisions
