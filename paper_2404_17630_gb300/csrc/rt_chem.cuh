@@ -231,6 +231,12 @@ __device__ __forceinline__ double largest_change(const double a[n], const double
   return f;
 }
 
+// x, and 0 where it is negative (NaN stays), on the integer pipe.
+__device__ __forceinline__ double clamp_neg(double x) {
+  const long long b = __double_as_longlong(x);
+  return b < 0 && (b & 0x7FFFFFFFFFFFFFFFLL) <= 0x7FF0000000000000LL ? 0.0 : x;
+}
+
 // One semi-implicit photochemistry attempt over dt from s into t; returns the
 // largest relative change f of the substep rule.  Steps: radiation level
 // over the step (implicit in N, absorbers at the start); photoionisation
@@ -295,10 +301,11 @@ __device__ double photochem_attempt(const ChemParams& P, double nH, double dt, c
           if (heat && (P.emask & (1 << (3 * b + q)))) ea = fma(P.eps[b][q], sn, ea);
         }
       if (heat) heat_e = fma(Nbar[b], ea, heat_e);
+      // N' = max(N - removed, 0); the flux by N' / N, by 0 where N <= 0 (the
+      // transport leaves slightly negative densities beside sharp fronts)
       double sc = fma(-(cdt * sum), inv[b], 1.0);
-      sc = __double_as_longlong(sc) > 0 ? sc : 0.0;
-      t.N[b] = s.N[b] * sc;
-      if (!(__double_as_longlong(s.N[b]) > 0)) sc = 0.0;
+      t.N[b] = clamp_neg(s.N[b] * sc);
+      if (!(__double_as_longlong(sc) > 0 && __double_as_longlong(s.N[b]) > 0)) sc = 0.0;
       t.f[b][0] = s.f[b][0] * sc;
       t.f[b][1] = s.f[b][1] * sc;
       t.f[b][2] = s.f[b][2] * sc;

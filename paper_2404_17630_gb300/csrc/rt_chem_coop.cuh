@@ -250,8 +250,13 @@ __device__ __forceinline__ auto group_attempt(const ChemParams& P, const Fit& fi
   // photons of the lane's bin: removed as the ionisations were credited
   const double suma = fma(g.sd[2], t.x[3], fma(g.sd[1], t.x[2], g.sd[0] * t.x[0]));
   double sc = fma(-(cdt * suma), inv1pt, 1.0);
-  sc = positive(sc) ? sc : 0.0;
-  t.N = s.N * sc;
+  if constexpr (Mixed) {
+    sc = positive(sc) ? sc : 0.0;
+    t.N = s.N * sc;
+  } else {
+    t.N = clamp_neg(s.N * sc);
+    sc = positive(sc) && positive(s.N) ? sc : 0.0;
+  }
   t.T = s.T;
   V f = V(0);
   // change of the lane's abundance (lanes 0-4)
@@ -280,7 +285,6 @@ __device__ __forceinline__ auto group_attempt(const ChemParams& P, const Fit& fi
 #pragma unroll
     for (int m = 1; m < 8; m <<= 1) f = fmaxf(f, xor_lane(f, m));
   } else {
-    if (!positive(s.N)) sc = 0.0;
     sc_out = sc;
     t.f = s.f * from_lane(sc, l < 9 ? l / 3 : 15);
     double fl = P.x_floor;
