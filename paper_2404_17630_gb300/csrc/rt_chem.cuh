@@ -237,6 +237,11 @@ __device__ __forceinline__ double clamp_neg(double x) {
   return b < 0 && (b & 0x7FFFFFFFFFFFFFFFLL) <= 0x7FF0000000000000LL ? 0.0 : x;
 }
 
+// |x| on the integer pipe.
+__device__ __forceinline__ double no_sign(double x) {
+  return __hiloint2double(__double2hiint(x) & 0x7FFFFFFF, __double2loint(x));
+}
+
 // One semi-implicit photochemistry attempt over dt from s into t; returns the
 // largest relative change f of the substep rule.  Steps: radiation level
 // over the step (implicit in N, absorbers at the start); photoionisation
@@ -447,10 +452,12 @@ __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double 
       for (int sp = 0; sp < 3; ++sp)
         if (P.smask & (1 << (3 * b + sp))) suma = fma(sg(b, sp), m[sp], suma);
       const double taup = IntCvt ? suma : cdt * suma;
+      // N' = max(N - removed, 0) and no flux where N <= 0, as in the FP64
+      // attempt: the factor is clamped on the integer pipe (a double's bits
+      // order like the value where it is positive), and a zero keeps no sign
       double sc = fma(-taup, inv1pt[b], 1.0);
-      // sc <- max(sc, 0) on the integer pipe (a double's bits order like
-      // the value where it is positive)
-      sc = __double_as_longlong(sc) > 0 ? sc : 0.0;
+      sc = __double_as_longlong(sc) > 0 && __double_as_longlong(s.N[b]) > 0 ? sc : 0.0;
+      t.N[b] = no_sign(s.N[b] * sc);
       if (heat) {
         float ea = 0.0f;
 #pragma unroll
@@ -458,7 +465,6 @@ __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double 
           if (P.emask & P.smask & (1 << (3 * b + sp))) ea = fmaf(P.heat_f[b][sp], mf[sp], ea);
         hsum = fmaf(to_f<IntCvt>(Nbar[b]), ea, hsum);
       }
-      t.N[b] = s.N[b] * sc;
       sc_out[b] = to_f<IntCvt>(sc);
     }
   }

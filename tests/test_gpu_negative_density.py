@@ -3,8 +3,8 @@ not keep N >= 0: a beam beside an almost empty region leaves small negative N, a
 larger ones without the limiter.  An attempt ends at max(N - removed, 0) and takes
 the flux of a cell with N <= 0 away.  Accepted first attempts, groups of lanes (216
 cells) and one thread per cell (50,653), whole steps, and the reverse mode, which
-differentiates the clamp.  Bounds as in the parity tests: 1e-12, reverse mode 1e-9,
-each against the oracle."""
+differentiates the clamp; in the mixed path too.  Bounds as in the parity tests: FP64
+1e-12, reverse mode 1e-9, mixed 1e-4, each against the oracle."""
 import numpy as np
 import pytest
 
@@ -104,3 +104,32 @@ def test_adjoint():
                     ("F", g["F"] * cfg["c_red"], ref["lam0"]["fr"]), ("x5", g["x5"], ref["lam0"]["x5"]),
                     ("T", g["T"], ref["lam0"]["T"])):
         assert np.abs(a - b).max() <= 1e-9 * np.abs(b).max(), k
+
+
+@pytest.mark.parametrize("n", [6, 37])
+def test_chemistry_mixed(n):
+    mesh, cfg, st = _negative(n)
+    o, rt = make_oracle(mesh, cfg, st), _gpu(mesh, cfg, st, precision="mixed", gather_sum=1)
+    dt = 0.9 * o.max_dt()
+    o.thermochemistry(dt)
+    rt.thermochemistry(dt)
+    rt.sync()
+    e = _errors(rt, o, cfg)
+    assert max(e.values()) < 1e-4, e
+
+
+def test_beam_mixed():
+    """One subcycle's chemistry on the state that the beam's FP64 transport leaves (N < 0 in it)."""
+    mesh, cfg, st = _beam(limiter=0)
+    o = make_oracle(mesh, cfg, st)
+    dt = 0.9 * o.max_dt()
+    for _ in range(8):
+        o.transport(dt)
+    N, fr = o.radiation()
+    assert N.min() < 0
+    rt = _gpu(mesh, cfg, dict(st, N=N, fr=fr), precision="mixed")
+    o.thermochemistry(dt)
+    rt.thermochemistry(dt)
+    rt.sync()
+    e = _errors(rt, o, cfg)
+    assert max(e.values()) < 1e-4, e
