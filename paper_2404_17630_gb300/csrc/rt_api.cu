@@ -527,7 +527,7 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   ar.add_bytes(&ctx->G, mx ? c * 4 * pad_bins(B) * sizeof(float4) : c * B * 12 * sizeof(double));
   ar.add_bytes(&ctx->flux, f * B * 4 * rs);
   ar.add_bytes(&ctx->hw, 2 * f * 4 * rs); ar.add_bytes(&ctx->hx, 2 * f * 4 * rs); ar.add_bytes(&ctx->xmax, c * rs);
-  ar.add(&ctx->work_cell, c); ar.add(&ctx->work_ctl, 4); ar.add(&ctx->ivol, c);
+  ar.add(&ctx->work_cell, c); ar.add(&ctx->work_ctl, kRestCtl); ar.add(&ctx->ivol, c);
   if (mx) {
     ar.add(&ctx->fa32, f); ar.add(&ctx->fb32, f); ar.add(&ctx->work_f1, c);
     ar.add(&ctx->shadow, c * B); ar.add(&ctx->radN, c * B);
@@ -603,7 +603,7 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
                                                             ctx->rL64, ctx->rR64, ctx->w64);
   }
   CK(cudaMemsetAsync(ctx->status, 0, sizeof(int), ctx->stream), "status");
-  CK(cudaMemsetAsync(ctx->work_ctl, 0, 4 * sizeof(int), ctx->stream), "worklist");
+  CK(cudaMemsetAsync(ctx->work_ctl, 0, kRestCtl * sizeof(int), ctx->stream), "worklist");
   k_geometry_cells<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->off, ctx->csr, ctx->w64, ctx->minv64, ctx->status);
   if (mx && F > 0) {
     k_build_facerecs<<<nblk(F), kThreads, 0, ctx->stream>>>(F, ctx->lr, ctx->nA64, ctx->rL64, ctx->rR64, ctx->fa32,

@@ -48,7 +48,7 @@ struct rt_ctx {
   int32_t* work_cell = nullptr;  // mixed chemistry worklist (cells whose first attempt was rejected)
   float* work_f1 = nullptr;
   double* work_f1d = nullptr;    // FP64 chemistry worklist: the rejected first attempt's measure
-  int* work_ctl = nullptr;       // entries, next entry, finished blocks (zero between subcycles)
+  int* work_ctl = nullptr;       // the worklist's counters (zero between subcycles)
   // individual time steps: the lists of the current active set (all null /
   // zero when every cell is active), a view of one entry of `sets`
   bool all_active = true;

@@ -1385,21 +1385,50 @@ __global__ void k_reciprocal(int n, const double* __restrict__ in, double* out) 
 // carry N and the gas only; the flux is read at the end and scaled by the
 // product of the accepted photon factors.
 
-// A worklist of at most this many cells goes to groups of lanes (rest_groups),
-// a longer one to one thread per cell (rest_threads): a group's attempt has a
-// third (FP64) or half (mixed) of the latency, but costs the FP64 unit several
-// times as much per cell, so that groups win while the longest chains decide.
-// Far from equilibrium (mean chain 11-47 attempts, longest 150-360), ms by
-// threads / by groups: FP64 4.2 / 1.3 at 991 cells, 5.7 / 2.4 at 12,035,
-// 8.8 / 6.2 at 32,006, 10.8 / 9.4 at 61,427; mixed 0.94 / 0.58, 1.29 / 0.98,
-// 1.89 / 1.90, 2.28 / 2.87.
+// The worklist's rule.  A group of lanes (rest_groups) makes an attempt in half
+// the latency of a thread (rest_threads): 17 k against 35 k cycles in FP64.  But
+// it costs the FP64 unit six times as much per cell, 6.4 k cycles against 1.1 k
+// in a full warp.  Groups therefore win while the longest chain of attempts
+// decides and lose where the list's whole work does: the line lies at a number
+// of chains side by side, (attempts of all cells) / (attempts of the longest),
+// of 2,700 in FP64 and 2,000 in the mixed path.  The chains are foretold by
+// their first attempts: a quantity that has to change by the measure f in steps
+// of f_s takes about ln(1 + f) / f_s of them.  The first pass adds these up and
+// keeps the largest (rest_entry), in integers, so that the choice does not
+// depend on the order of the list.  Foretold so, the line lies at 2,000 and
+// 1,500.  ms by threads / by groups at (cells; foretold chains side by side):
+// FP64 4.06 / 2.54 (12,074; 1,186), 10.6 / 11.8 (12,147; 1,853), 4.38 / 4.43
+// (34,535; 2,575), 9.04 / 20.6 (21,511; 10,121), and for even chains 0.135 /
+// 0.41 (12,167; 11,701); mixed 1.22 / 0.96, 3.16 / 3.62, 1.26 / 1.39, 2.53 / 5.75,
+// 0.047 / 0.137.  Beyond the lengths below the sums are not looked at.
 constexpr int kGroupMax64 = 49152, kGroupMaxMixed = 24576;
+constexpr int kGroupSide64 = 2000, kGroupSideMixed = 1500;
 
-// Worklist of the cells whose first attempt was rejected.
+// Entry of a rejected cell with measure f1 in the worklist whose counters are
+// ctl: its place.  One addition per warp and counter.
+__device__ __forceinline__ int rest_entry(int* ctl, float f1) {
+  const int k = atomicAdd(ctl, 1);
+  const int w = 1 + (int)(1000.0f * fminf(__log2f(1.0f + f1), 32.0f));   // 49,152 of them fit the sum
+  const unsigned m = __activemask();
+  const int sum = __reduce_add_sync(m, w), top = __reduce_max_sync(m, w);
+  if ((int)(threadIdx.x & 31) == __ffs(m) - 1) {
+    atomicAdd(ctl + 1, sum);
+    atomicMax(ctl + 2, top);
+  }
+  return k;
+}
+__device__ __forceinline__ bool rest_by_groups(const int4& c, int most, int side) {
+  return c.x <= most && c.y <= side * c.z;
+}
+
+// Worklist of the cells whose first attempt was rejected, and its counters:
+// entries, sum and largest of the foretold chains (read together, as one
+// 16-byte word), next entry to hand out, finished warps.
+constexpr int kRestCtl = 5, kRestNext = 3, kRestDone = 4;
 struct ChemWork {
   int32_t* cell;   // C
   float* f1;       // C: the rejected first attempt's measure
-  int* ctl;        // [0] entries, [1] next entry to hand out, [2] finished blocks
+  int* ctl;        // kRestCtl counters
 };
 
 // Source term of Eq. (E) over the subcycle: the photons of the cell's
@@ -1476,7 +1505,7 @@ __global__ void __launch_bounds__(128, 6) k_chem_first(CellArgs a, ChemParams P,
 #pragma unroll
   for (int b = 0; b < kMaxBins; ++b)
     if (b < a.B) a.radN[(size_t)i * a.B + b] = s.N[b];
-  const int k = atomicAdd(w.ctl, 1);
+  const int k = rest_entry(w.ctl, f1);
   w.cell[k] = i;
   w.f1[k] = f1;
 }
@@ -1487,8 +1516,8 @@ __device__ __forceinline__ void rest_done(int* ctl) {
   __syncwarp();
   if ((threadIdx.x & 31) == 0) {
     __threadfence();
-    if (atomicAdd(ctl + 2, 1) == (int)(gridDim.x * (blockDim.x >> 5)) - 1) {
-      ctl[0] = ctl[1] = ctl[2] = 0;
+    if (atomicAdd(ctl + kRestDone, 1) == (int)(gridDim.x * (blockDim.x >> 5)) - 1) {
+      for (int q = 0; q < kRestCtl; ++q) ctl[q] = 0;
       __threadfence();
     }
   }
@@ -1502,7 +1531,7 @@ __device__ __forceinline__ int group_first() {
 }
 __device__ __forceinline__ int group_next(int* ctl, bool need, int l) {
   int k = 0;
-  if (need && l == 0) k = (int)(gridDim.x * (blockDim.x / kGroup)) + atomicAdd(ctl + 1, 1);
+  if (need && l == 0) k = (int)(gridDim.x * (blockDim.x / kGroup)) + atomicAdd(ctl + kRestNext, 1);
   return from_lane(k, 0);
 }
 
@@ -1612,17 +1641,17 @@ __device__ __forceinline__ void rest_threads(const CellArgs& a, const ChemParams
       chem_store_mixed(a, i, s, S, n, true, shadow);
     }
     int next = 0;
-    if (lane == 0) next = n_warps + atomicAdd(w.ctl + 1, 1);
+    if (lane == 0) next = n_warps + atomicAdd(w.ctl + kRestNext, 1);
     chunk = __shfl_sync(0xffffffffu, next, 0);
   }
 }
 
 __global__ void __launch_bounds__(128) k_chem_rest(CellArgs a, ChemParams P, float4* __restrict__ shadow,
                                                    ChemWork w) {
-  const int total = *(volatile int*)w.ctl;
-  if (total == 0) return;   // nothing was rejected: the worklist's counters are all zero already
-  if (total <= kGroupMaxMixed) rest_groups(a, P, shadow, w, total);
-  else rest_threads(a, P, shadow, w, total);
+  const int4 c = *reinterpret_cast<const int4*>(w.ctl);
+  if (c.x == 0) return;   // nothing was rejected: the worklist's counters are all zero already
+  if (rest_by_groups(c, kGroupMaxMixed, kGroupSideMixed)) rest_groups(a, P, shadow, w, c.x);
+  else rest_threads(a, P, shadow, w, c.x);
   rest_done(w.ctl);
 }
 
@@ -1752,7 +1781,7 @@ __global__ void __launch_bounds__(128) k_chem64_first(CellArgs a, ChemParams P, 
 #pragma unroll
   for (int b = 0; b < kMaxBins; ++b)
     if (b < a.B) a.rad[(size_t)i * a.B + b].x = s.N[b];
-  const int k = atomicAdd(work_ctl, 1);
+  const int k = rest_entry(work_ctl, (float)f1);
   work_cell[k] = i;
   work_f1[k] = f1;
 }
@@ -1913,7 +1942,7 @@ __device__ __forceinline__ void rest_threads64(const CellArgs& a, const ChemPara
       chem_store64(a, i, s, true);
     }
     int next = 0;
-    if (lane == 0) next = n_warps + atomicAdd(work_ctl + 1, 1);
+    if (lane == 0) next = n_warps + atomicAdd(work_ctl + kRestNext, 1);
     chunk = __shfl_sync(0xffffffffu, next, 0);
   }
 }
@@ -1922,10 +1951,11 @@ template <bool kTape>
 __global__ void __launch_bounds__(128) k_chem64_rest(CellArgs a, ChemParams P, const int32_t* __restrict__ work_cell,
                                                      const double* __restrict__ work_f1, int* work_ctl,
                                                      ChemTape tape) {
-  const int total = *(volatile int*)work_ctl;
-  if (total == 0) return;   // nothing was rejected: the worklist's counters are all zero already
-  if (total <= kGroupMax64) rest_groups64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, total);
-  else rest_threads64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, total);
+  const int4 c = *reinterpret_cast<const int4*>(work_ctl);
+  if (c.x == 0) return;   // nothing was rejected: the worklist's counters are all zero already
+  if (rest_by_groups(c, kGroupMax64, kGroupSide64))
+    rest_groups64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, c.x);
+  else rest_threads64<kTape>(a, P, work_cell, work_f1, work_ctl, tape, c.x);
   rest_done(work_ctl);
 }
 
