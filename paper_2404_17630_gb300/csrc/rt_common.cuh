@@ -136,6 +136,17 @@ __device__ __forceinline__ double f2d_int(float f) {
   return __hiloint2double((int)(sign | ((e + 896u) << 20) | (m >> 3)), (int)(m << 29));
 }
 
+// f2d_int for every float: values below 1 are scaled by 2^64 first, which makes
+// the subnormal ones normal and changes no other bit.
+__device__ __forceinline__ double f2d_all(float f) {
+  const bool small = fabsf(f) < 1.0f;
+  const unsigned b = __float_as_uint(small ? f * 0x1p64f : f);
+  const unsigned sign = b & 0x80000000u, e = (b >> 23) & 0xFFu, m = b & 0x7FFFFFu;
+  if (e == 0u) return __hiloint2double((int)sign, 0);
+  if (e == 255u) return __hiloint2double((int)(sign | 0x7FF00000u | (m ? 0x80000u : 0u)), 0);
+  return __hiloint2double((int)(sign | ((e + (small ? 832u : 896u)) << 20) | (m >> 3)), (int)(m << 29));
+}
+
 // x is infinite or NaN: all exponent bits set (an integer test; the FP64
 // pipe's comparison is left free).
 __device__ __forceinline__ bool nonfinite_bits(double x) {

@@ -1250,7 +1250,8 @@ __device__ __forceinline__ void flux_sum(const CellArgs& a, const R4<R>* __restr
   // rounding: the same sum as the add or subtract, without predicated copies
   // of both).  FP32 terms: the sign set and the term widened on the integer
   // pipe (the FP64 unit, which bounds this sum, also executes the hardware's
-  // conversion: 66 -> 40 us at 64,000 cells and three bins).
+  // conversion: 66 -> 42 us at 64,000 cells and three bins), subnormal terms
+  // included: with N near 1e-37 many are.
   auto add = [&](int e, const R4<R>& v) {
     if constexpr (sizeof(R) == 8) {
       const double sg = (e & 1) ? -1.0 : 1.0;
@@ -1260,10 +1261,10 @@ __device__ __forceinline__ void flux_sum(const CellArgs& a, const R4<R>* __restr
       acc[3] = fma(sg, v.w, acc[3]);
     } else {
       const unsigned sg = (unsigned)(e & 1) << 31;
-      acc[0] += f2d_int(__uint_as_float(__float_as_uint(v.x) ^ sg));
-      acc[1] += f2d_int(__uint_as_float(__float_as_uint(v.y) ^ sg));
-      acc[2] += f2d_int(__uint_as_float(__float_as_uint(v.z) ^ sg));
-      acc[3] += f2d_int(__uint_as_float(__float_as_uint(v.w) ^ sg));
+      acc[0] += f2d_all(__uint_as_float(__float_as_uint(v.x) ^ sg));
+      acc[1] += f2d_all(__uint_as_float(__float_as_uint(v.y) ^ sg));
+      acc[2] += f2d_all(__uint_as_float(__float_as_uint(v.z) ^ sg));
+      acc[3] += f2d_all(__uint_as_float(__float_as_uint(v.w) ^ sg));
     }
   };
   int k = k0;
