@@ -696,19 +696,24 @@ rt_status rt_set_sources(rt_ctx* ctx, int64_t n, const int64_t* cell, const doub
     CK(cudaMemcpy(hq.data(), Q, n * B * 8, is_device_ptr(Q) ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost),
        "sources");
   }
-  // bin rates per cell, summed in source order
+  // bin rates per cell, summed in source order.  The index of a cell: from an
+  // array over the cells where there are many sources, which costs 0.1 ms per
+  // million cells, else from a map, which costs 0.1 to 0.2 us per source
+  // (200,000 sources in a million cells: 39 ms by the map, 4.3 by the array).
   std::unordered_map<int64_t, int> index;
+  std::vector<int32_t> dense(n > ctx->C / 256 ? ctx->C : 0, -1);
   std::vector<int32_t> where;
   std::vector<double> rate;
   for (int64_t k = 0; k < n; ++k) {
     if (hc[k] < 0 || hc[k] >= ctx->C) return fail(ctx, RT_INVALID_ARG, "source %lld in cell %lld out of range",
                                                   (long long)k, (long long)hc[k]);
-    const auto it = index.try_emplace(hc[k], (int)where.size());
-    if (it.second) {
+    int& i = dense.empty() ? index.try_emplace(hc[k], -1).first->second : dense[hc[k]];
+    if (i < 0) {
+      i = (int)where.size();
       where.push_back((int32_t)hc[k]);
       rate.resize(where.size() * B, 0.0);
     }
-    for (int b = 0; b < B; ++b) rate[(size_t)it.first->second * B + b] += hq[(size_t)k * B + b];
+    for (int b = 0; b < B; ++b) rate[(size_t)i * B + b] += hq[(size_t)k * B + b];
   }
   const int m = (int)where.size();
   if (m > ctx->src_cap) {
