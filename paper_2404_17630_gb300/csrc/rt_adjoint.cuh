@@ -41,20 +41,18 @@ __device__ __forceinline__ d4 adj_side(const d4& p, const double* __restrict__ G
   const double e3 = fma(c.y, x.x, fma(c.z, x.y, fma(c.w, x.z, p.w)));
   const bool clampN = lt_zero(e0);
   const double N = clampN ? 0.0 : e0, N2 = N * N, q2 = e1 * e1 + e2 * e2 + e3 * e3;
-  const bool clampF = gt_nonneg(q2, N2);
+  const bool over = nonfinite_bits(q2), clampF = gt_nonneg(q2, N2) || over;
   double F1 = e1, F2 = e2, F3 = e3, fl2 = q2;
   double ifl = 0.0;
   if (clampF) {
     ifl = div_nr(1.0, sqrt_nr(q2));
     const double r = N * ifl;
     F1 *= r; F2 *= r; F3 *= r;
-    fl2 = N2;
+    fl2 = over ? 0.0 : N2;
   }
   double lf1 = l0[0], lf2 = l0[1], lf3 = l0[2];
   if (gt_nonneg(N, 0.0) && gt_nonneg(fl2, 0.0)) {
-    double t = fma(-3.0, fl2, 4.0 * N2);
-    t = gt_nonneg(N2, t) ? N2 : t;
-    const double s = sqrt_nr(t), d = fma(2.0, N, s);
+    const double s = m1_root(N, N2, fl2), d = fma(2.0, N, s);
     // (one reciprocal of d s would leave the exponent range at densities that
     // occur beyond a light front: N^2 < 1e-308)
     const double id3 = 3.0 * rcp_nr<2>(d), is = rcp_nr<2>(s);

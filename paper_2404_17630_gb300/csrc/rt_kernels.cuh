@@ -999,11 +999,27 @@ __device__ __forceinline__ void face_state(const d4& p, const double* __restrict
   if (lt_zero(v[0])) v[0] = 0.0;
   N2 = v[0] * v[0];
   fl2 = v[1] * v[1] + v[2] * v[2] + v[3] * v[3];
-  if (gt_nonneg(fl2, N2)) {
+  const bool over = nonfinite_bits(fl2);   // |F| beyond 1e154: F = 0, as by the definition's own squares
+  if (gt_nonneg(fl2, N2) || over) {
     const double s = div_nr(v[0], sqrt_nr(fl2));
     v[1] *= s; v[2] *= s; v[3] *= s;
-    fl2 = N2;
+    fl2 = over ? 0.0 : N2;
   }
+}
+
+// s = sqrt(4 N^2 - 3 |F|^2) >= N within rounding (f <= 1), from the squares; where
+// N^2 is near an end of the exponent range (densities beyond 1e150 or below
+// 1e-150), from squares scaled by a power of two.
+__device__ __forceinline__ double m1_root(double N, double N2, double fl2) {
+  const unsigned e = (unsigned)__double2hiint(N2) & 0x7FF00000u;
+  if (e - (23u << 20) < (2000u << 20)) {   // 2^-1000 <= N^2 < 2^1000
+    const double t = fma(-3.0, fl2, 4.0 * N2);
+    return sqrt_nr(gt_nonneg(N2, t) ? N2 : t);
+  }
+  const bool big = e >= 0x40000000u;
+  const double c = big ? 0x1p-600 : 0x1p600, n = N * c, n2 = n * n;
+  const double t = fma(-3.0, fl2 * c * c, 4.0 * n2);
+  return sqrt_nr(gt_nonneg(n2, t) ? n2 : t) * (big ? 0x1p600 : 0x1p-600);
 }
 
 // The same extrapolation from the four groups of an FP32 gradient record:
@@ -1053,8 +1069,7 @@ __device__ __forceinline__ void m1_normal(const float v[4], float n0, float n1, 
 // where N is small.  The kernel is bound by the FP64 unit: 1.67 -> 0.96 ms per
 // launch at 250,047 cells, 234 -> 138 us at 262,144 cells with one bin (1.06 and
 // 0.152 with the squares formed twice).
-// Here: the two coefficients of 3 N D n = a n + 9 k F, and F . n.  s >= N
-// (f <= 1, also where the squares are rounded or leave the normal range).
+// Here: the two coefficients of 3 N D n = a n + 9 k F, and F . n.
 __device__ __forceinline__ void m1_coef(const double v[4], double N2, double fl2, double n0, double n1, double n2,
                                         double& a, double& k, double& un) {
   un = v[1] * n0 + v[2] * n1 + v[3] * n2;
@@ -1062,9 +1077,7 @@ __device__ __forceinline__ void m1_coef(const double v[4], double N2, double fl2
   k = 0.0;
   // the tests on the integer pipe (v[0] >= 0 after the face-state clamp)
   if (gt_nonneg(v[0], 0.0) && gt_nonneg(fl2, 0.0)) {
-    double t = fma(-3.0, fl2, 4.0 * N2);
-    t = __double_as_longlong(N2) > __double_as_longlong(t) ? N2 : t;
-    const double s = sqrt_nr(t);
+    const double s = m1_root(v[0], N2, fl2);
     a = s - v[0];
     k = div_nr(un, fma(2.0, v[0], s));
   }
