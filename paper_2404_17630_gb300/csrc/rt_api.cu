@@ -200,14 +200,14 @@ rt_status check_config(const rt_config* c) {
 template <class R> Geo<R> geo(const rt_ctx* ctx);
 template <> Geo<double> geo<double>(const rt_ctx* c) {
   return Geo<double>{c->C, c->F, c->B, make_divb(c->B), c->off, c->csr, c->nbr, c->lr, c->nA64, c->rL64, c->rR64,
-                     (const d4*)c->hw, (const d4*)c->hx, c->hx32, (const double*)c->xmax, nullptr, nullptr, c->B,
+                     (const d4*)c->hw, (const d4*)c->hx, c->hx32, c->xm32, (const double*)c->xmax, nullptr, nullptr, c->B,
                      c->touched_cells, c->n_touched,
                      c->grad_blocks, c->n_grad_blocks, c->touched, c->act_faces, c->n_act_faces};
 }
 template <> Geo<float> geo<float>(const rt_ctx* c) {
   // the FP32 sweep reads faces through fa / fb; no per-array face copies
   return Geo<float>{c->C, c->F, c->B, make_divb(c->B), c->off, c->csr, c->nbr, c->lr, nullptr, nullptr, nullptr,
-                    (const float4*)c->hw, (const float4*)c->hx, nullptr, (const float*)c->xmax, c->fa32, c->fb32,
+                    (const float4*)c->hw, (const float4*)c->hx, nullptr, nullptr, (const float*)c->xmax, c->fa32, c->fb32,
                     pad_bins(c->B),
                     c->touched_cells, c->n_touched, c->grad_blocks, c->n_grad_blocks, c->touched, c->act_faces,
                     c->n_act_faces};
@@ -533,6 +533,7 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
     ar.add(&ctx->shadow, c * B); ar.add(&ctx->radN, c * B);
   } else {
     ar.add(&ctx->rad, c * B); ar.add(&ctx->work_f1d, c); ar.add(&ctx->hx32, 2 * f);
+    ar.add(&ctx->xm32, c);
   }
   {
     void* p = nullptr;
@@ -611,19 +612,19 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   }
   k_reciprocal<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->vol, ctx->ivol);
   if (F > 0) {
-    if (mx)
+    if (mx) {
       k_build_halfedges<float><<<nblk(2LL * F), kThreads, 0, ctx->stream>>>(
           2 * F, ctx->csr, ctx->nbr, ctx->lr, ctx->minv64, ctx->w64, ctx->rL64, ctx->rR64, (float4*)ctx->hw,
-          (float4*)ctx->hx, nullptr);
-    else
-      k_build_halfedges<double><<<nblk(2LL * F), kThreads, 0, ctx->stream>>>(
-          2 * F, ctx->csr, ctx->nbr, ctx->lr, ctx->minv64, ctx->w64, ctx->rL64, ctx->rR64, (d4*)ctx->hw, (d4*)ctx->hx,
-          ctx->hx32);
-    if (mx)
+          (float4*)ctx->hx);
       k_cell_xmax<float><<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->off, (const float4*)ctx->hx,
                                                                (float*)ctx->xmax);
-    else
+    } else {
+      k_build_halfedges<double><<<nblk(2LL * F), kThreads, 0, ctx->stream>>>(
+          2 * F, ctx->csr, ctx->nbr, ctx->lr, ctx->minv64, ctx->w64, ctx->rL64, ctx->rR64, (d4*)ctx->hw, (d4*)ctx->hx);
       k_cell_xmax<double><<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->off, (const d4*)ctx->hx, (double*)ctx->xmax);
+      k_cell_search<<<nblk(C), kThreads, 0, ctx->stream>>>(C, ctx->off, (const d4*)ctx->hx, (const double*)ctx->xmax,
+                                                           ctx->hx32, ctx->xm32);
+    }
   }
   if ((st = launched(ctx, "geometry kernels"))) return wait_fail(ctx, st);
   int h_status = 0;

@@ -322,7 +322,8 @@ template <class R> struct Geo {
   const R4<R>* rR;        // F: x_f - s_R
   const R4<R>* hw;        // 2F half-edges in CSR order: (+- M^-1 w, sign + for the left cell; neighbour id bits)
   const R4<R>* hx;        // 2F half-edges in CSR order: x_f - s of this cell's side
-  const float4* hx32;     // FP64 sweep: the offsets of hx in FP32
+  const float4* hx32;     // FP64 sweep: the offsets of hx in FP32, scaled per cell
+  const float* xm32;      // FP64 sweep, C: the largest |x| in that scale
   const R* xmax;          // C: max over the cell's half-edges of hx.w (|x| in FP32, |x|^2 in FP64)
   const f8* fa;           // FP32 sweep, F: (n, A, x_f - s_L, left id bits)
   const float4* fb;       // FP32 sweep, F: (x_f - s_R, right id bits)

@@ -27,7 +27,8 @@ struct rt_ctx {
   int2* lr = nullptr;
   d4 *nA64 = nullptr, *rL64 = nullptr, *rR64 = nullptr, *w64 = nullptr;
   void *hw = nullptr, *hx = nullptr;   // half-edge records in the sweep precision
-  float4* hx32 = nullptr;              // FP64 sweep: the half-edges' offsets in FP32
+  float4* hx32 = nullptr;              // FP64 sweep: the half-edges' offsets in FP32, scaled per cell
+  float* xm32 = nullptr;               // and per cell the largest of their lengths
   void* xmax = nullptr;                 // per cell: the largest .w of its offset records (sweep precision)
   double* minv64 = nullptr;
   // FP32 copies (mixed precision)

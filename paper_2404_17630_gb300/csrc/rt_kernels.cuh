@@ -284,13 +284,12 @@ __global__ void k_geometry_cells(int C, const int32_t* __restrict__ off, const i
 // 36 operations and six loads less per (cell, bin)), the neighbour id, and the
 // face-centre offset x from this cell with, in the fourth lane, |x| (FP32
 // sweep) or |x|^2 (FP64 sweep, summed in the order of the limiter's
-// definition) for the limiter's regularisation test.  FP64 sweep: the offset
-// in FP32 as well (hx32, for the limiter's search).
+// definition) for the limiter's regularisation test.
 template <class R>
 __global__ void k_build_halfedges(int n, const int32_t* __restrict__ csr, const int32_t* __restrict__ nbr,
                                   const int2* __restrict__ lr, const double* __restrict__ minv,
                                   const d4* __restrict__ w, const d4* __restrict__ rL, const d4* __restrict__ rR,
-                                  R4<R>* hw, R4<R>* hx, float4* hx32) {
+                                  R4<R>* hw, R4<R>* hx) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const int e = csr[k], f = e >> 1;
@@ -309,7 +308,6 @@ __global__ void k_build_halfedges(int n, const int32_t* __restrict__ csr, const 
   b.x = (R)x.x; b.y = (R)x.y; b.z = (R)x.z;
   b.w = sizeof(R) == 4 ? (R)sqrt(xx) : (R)xx;
   hx[k] = b;
-  if (hx32) hx32[k] = make_float4((float)x.x, (float)x.y, (float)x.z, 0.f);
 }
 
 // Per cell, the largest hx.w over its half-edges (|x| in FP32, |x|^2 in FP64):
@@ -324,6 +322,28 @@ __global__ void k_cell_xmax(int C, const int32_t* __restrict__ off, const R4<R>*
     m = w > m ? w : m;
   }
   xmax[i] = m;
+}
+
+// FP64 sweep, per cell, for the limiter's search: the offsets in FP32, scaled by a
+// power of two of the cell's own so that the largest |x_f| lies in [1, 2) whatever
+// the unit of length (with cells of 1e20 cm unscaled offsets left FP32's range, and
+// the search came on top of the scan it was to spare: 251 us a launch instead of
+// 167 at 64,000 cells and three bins), and that largest |x_f|, NaN where |x_f|^2 is
+// not a normal number.
+__global__ void k_cell_search(int C, const int32_t* __restrict__ off, const d4* __restrict__ hx,
+                              const double* __restrict__ xmax, float4* __restrict__ hx32, float* __restrict__ xm32) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= C) return;
+  const double X = xmax[i];
+  const int e = (__double2hiint(X) >> 20) - 1023;   // X > 0: in [-1022, 1023] where it is normal
+  const bool ok = e >= -1022 && e <= 1023;
+  const int k = ok ? e >> 1 : 0;
+  const double s = __hiloint2double((1023 - k) << 20, 0);   // 2^-k
+  for (int q = off[i]; q < off[i + 1]; ++q) {
+    const d4 x = hx[q];
+    hx32[q] = make_float4((float)(x.x * s), (float)(x.y * s), (float)(x.z * s), 0.f);
+  }
+  xm32[i] = ok ? sqrtf((float)(X * s * s)) : nanf("");
 }
 
 // Face records of the FP32 sweep: (n, A, x_f - s_L, left id) in 32 bytes
@@ -666,7 +686,7 @@ __global__ void __launch_bounds__(256) k_grad(Geo<R> g, const R4<R>* __restrict_
         eg[q] = sqrtf(lim_eps2 * (gr[q][0] * gr[q][0] + gr[q][1] * gr[q][1] + gr[q][2] * gr[q][2]));
       lim_extremes(g.hx, k0, k1, gr, eg, __ldg(g.xmax + i), dpos, dneg);
     } else {
-      lim_extremes(g.hx, g.hx32, k0, k1, gr, lim_eps2, __ldg(g.xmax + i), dpos, dneg, at);
+      lim_extremes(g.hx, g.hx32, k0, k1, gr, lim_eps2, __ldg(g.xmax + i), __ldg(g.xm32 + i), dpos, dneg, at);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {

@@ -61,24 +61,25 @@ __device__ __forceinline__ bool scaled_f32(const double g[3], float o[3]) {
 // dneg = min(0, min g.x_f) over the faces k0..k1-1 that pass the
 // regularisation test (g.x_f)^2 > eps2 |g|^2 |x_f|^2 (X: the largest x.w =
 // |x_f|^2), kept as bit patterns (integer compares; the FP64 pipe is the
-// kernel's bound).  First a search in FP32 for the face that attains each
-// extreme: |g| scaled to below 2 per component, the FP32 product g . x_f is
-// within 6 2^-24 2 (|x| + |y| + |z|) <= 1.3e-6 |x_f| of the exact one (both
-// operands rounded, three roundings of the sum), so a leader that is 2.6e-6 of
-// the cell's largest |x_f| ahead of every other face and of zero is the FP64
-// leader, and its FP64 product is the extreme: eight FP64 products per (cell,
-// bin) instead of four per face (with the matrix folded into the weights:
-// 0.85 -> 0.52 ms per launch at 250,047 cells, 142 -> 82 us at 262,144 cells of six
-// faces and one bin).  A leader beyond the test's bound
-// for the largest |x_f|, by the same margin, also passes its own test, and
-// nothing more is to be tested: rounding is monotone.  Where a lead is smaller
+// kernel's bound).  xf: the offsets in FP32, in any unit that is the same for the
+// cell's faces, xm: the largest |x_f| in it (NaN: no search).  First a search in
+// FP32 for the face that attains each extreme: |g| scaled to below 2 per
+// component, the FP32 product g . x_f is within 6 2^-24 2 (|x| + |y| + |z|) <=
+// 1.3e-6 |x_f| of the exact one (both operands rounded, three roundings of the
+// sum), so a leader that is 2.6e-6 of the cell's largest |x_f| ahead of every
+// other face and of zero is the FP64 leader, and its FP64 product is the
+// extreme: eight FP64 products per (cell, bin) instead of four per face (with
+// the matrix folded into the weights: 0.85 -> 0.52 ms per launch at 250,047
+// cells, 142 -> 82 us at 262,144 cells of six faces and one bin).  A leader
+// beyond the test's bound for the largest |x_f|, by the same margin, also passes
+// its own test, and nothing more is to be tested: rounding is monotone.  Where a lead is smaller
 // (faces that tie by symmetry; a leader within the band of zero) every face's
 // product is formed in FP64 and, where an extreme does not clear the bound,
 // tested.  A component without gradient has no extremes.  at[2q], at[2q + 1]: the
 // first face that attains dpos[q], dneg[q].
 __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const float4* __restrict__ xf, int k0, int k1,
-                                             const double gr[4][3], double eps2, double X, double dpos[4],
-                                             double dneg[4], int at[8]) {
+                                             const double gr[4][3], double eps2, double X, float xm,
+                                             double dpos[4], double dneg[4], int at[8]) {
   float gf[4][3], m1[8], m2[8];
   bool flat[4], sure = true;
 #pragma unroll
@@ -105,8 +106,6 @@ __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const fl
       }
     }
   }
-  const float xm = sqrtf((float)X);
-  sure = sure && xm > 1e-18f && xm < 1e18f;
   const float ex = 1.0001f * sqrtf((float)eps2) * xm, lead = 2.6e-6f * xm;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {

@@ -90,8 +90,9 @@ constexpr size_t kNaSmem = kNaCap * (2 * sizeof(d4) + sizeof(float4)) + kNaCells
 // FP64 unit (about 1.7 k FP64 instructions per cell of 15.4 faces and three
 // bins; with the geometry formed per bin and per pass, its divisions and the
 // limiter's quotient per face and component 13 k): 3.22 -> 0.39 ms at 91,125
-// cells.  A block whose cells have
-// more than kNaCap half-edges forms them anew at each use.
+// cells.  With lengths beyond 1e18 or below 1e-18 the limiter does without its
+// FP32 search: 281 -> 371 us at 64,000 cells.  A block whose cells have more
+// than kNaCap half-edges forms them anew at each use.
 __global__ void __launch_bounds__(kNaCells * 3) k_noalloc_grad(NoallocArgs a) {
   extern __shared__ __align__(32) unsigned char smem[];
   d4* sw = reinterpret_cast<d4*>(smem);
@@ -185,7 +186,10 @@ __global__ void __launch_bounds__(kNaCells * 3) k_noalloc_grad(NoallocArgs a) {
     double dpos[4], dneg[4];
     if (staged) {
       int at[8];
-      lim_extremes(sx, sf, k0 - kb, k1 - kb, g, a.lim_eps2, __longlong_as_double(X), dpos, dneg, at);
+      // offsets that FP32 holds, with their squares (in cm a cell of 1e19 does not: every face's product in FP64)
+      float xm = sqrtf((float)__longlong_as_double(X));
+      if (!(xm > 1e-18f && xm < 1e18f)) xm = nanf("");
+      lim_extremes(sx, sf, k0 - kb, k1 - kb, g, a.lim_eps2, __longlong_as_double(X), xm, dpos, dneg, at);
     } else {
       long long p[4] = {0, 0, 0, 0}, q4[4] = {0, 0, 0, 0};
       double thr[4];
