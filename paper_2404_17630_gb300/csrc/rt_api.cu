@@ -450,61 +450,8 @@ rt_status need_mesh(rt_ctx* ctx) {
   return RT_OK;
 }
 
-}  // namespace
-
-// ===========================================================================
-// C ABI
-// ===========================================================================
-
-extern "C" {
-
-rt_status rt_create(const rt_config* cfg, void* stream, rt_ctx** out) {
-  if (!out) return fail(nullptr, RT_INVALID_ARG, "out is NULL");
-  *out = nullptr;
-  if (!cfg) return fail(nullptr, RT_INVALID_ARG, "cfg is NULL");
-  rt_status st = check_config(cfg);
-  if (st) return st;
-  rt_ctx* ctx = new rt_ctx;
-  ctx->cfg = *cfg;
-  ctx->stream = (cudaStream_t)stream;
-  ctx->B = cfg->n_bins;
-  cudaError_t e = cudaGetDevice(&ctx->device);
-  if (e != cudaSuccess) {
-    delete ctx;
-    cudaGetLastError();
-    return fail(nullptr, RT_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
-  }
-  if (cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
-      ctx->n_sm < 1) {
-    cudaGetLastError();
-    ctx->n_sm = 1;
-  }
-  int l2 = 0;
-  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->device) != cudaSuccess || l2 < 0) {
-    cudaGetLastError();
-    l2 = 0;
-  }
-  ctx->l2_bytes = (size_t)l2;
-  *out = ctx;
-  return RT_OK;
-}
-
-rt_status rt_set_stream(rt_ctx* ctx, void* stream) {
-  if (!ctx) return fail(nullptr, RT_INVALID_ARG, "null context");
-  ctx->stream = (cudaStream_t)stream;
-  ctx->gen++;
-  return RT_OK;
-}
-
-rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces) {
-  if (!ctx) return fail(nullptr, RT_INVALID_ARG, "null context");
-  if (!cells || !faces) return fail(ctx, RT_INVALID_ARG, "cells or faces is NULL");
-  if (cells->n <= 0 || faces->n < 0 || cells->n > (1LL << 30) || faces->n > (1LL << 29))
-    return fail(ctx, RT_INVALID_ARG, "cell or face count out of range");
-  if (!cells->volume || !cells->cx || !cells->cy || !cells->cz || !faces->left || !faces->right || !faces->area ||
-      !faces->nx || !faces->ny || !faces->nz || !faces->fx || !faces->fy || !faces->fz)
-    return fail(ctx, RT_INVALID_ARG, "mesh array is NULL");
-  free_all(ctx);
+// rt_init_mesh after the checks of its arguments, on a context without a mesh.
+rt_status build_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces) {
   const int C = (int)cells->n, F = (int)faces->n, B = ctx->B;
   ctx->C = C;
   ctx->F = F;
@@ -653,6 +600,66 @@ rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces
   ctx->n_src_cells = 0;
   ctx->mesh_ready = true;
   return RT_OK;
+}
+
+}  // namespace
+
+// ===========================================================================
+// C ABI
+// ===========================================================================
+
+extern "C" {
+
+rt_status rt_create(const rt_config* cfg, void* stream, rt_ctx** out) {
+  if (!out) return fail(nullptr, RT_INVALID_ARG, "out is NULL");
+  *out = nullptr;
+  if (!cfg) return fail(nullptr, RT_INVALID_ARG, "cfg is NULL");
+  rt_status st = check_config(cfg);
+  if (st) return st;
+  rt_ctx* ctx = new rt_ctx;
+  ctx->cfg = *cfg;
+  ctx->stream = (cudaStream_t)stream;
+  ctx->B = cfg->n_bins;
+  cudaError_t e = cudaGetDevice(&ctx->device);
+  if (e != cudaSuccess) {
+    delete ctx;
+    cudaGetLastError();
+    return fail(nullptr, RT_CUDA, "cudaGetDevice: %s", cudaGetErrorString(e));
+  }
+  if (cudaDeviceGetAttribute(&ctx->n_sm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
+      ctx->n_sm < 1) {
+    cudaGetLastError();
+    ctx->n_sm = 1;
+  }
+  int l2 = 0;
+  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, ctx->device) != cudaSuccess || l2 < 0) {
+    cudaGetLastError();
+    l2 = 0;
+  }
+  ctx->l2_bytes = (size_t)l2;
+  *out = ctx;
+  return RT_OK;
+}
+
+rt_status rt_set_stream(rt_ctx* ctx, void* stream) {
+  if (!ctx) return fail(nullptr, RT_INVALID_ARG, "null context");
+  ctx->stream = (cudaStream_t)stream;
+  ctx->gen++;
+  return RT_OK;
+}
+
+rt_status rt_init_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces) {
+  if (!ctx) return fail(nullptr, RT_INVALID_ARG, "null context");
+  if (!cells || !faces) return fail(ctx, RT_INVALID_ARG, "cells or faces is NULL");
+  if (cells->n <= 0 || faces->n < 0 || cells->n > (1LL << 30) || faces->n > (1LL << 29))
+    return fail(ctx, RT_INVALID_ARG, "cell or face count out of range");
+  if (!cells->volume || !cells->cx || !cells->cy || !cells->cz || !faces->left || !faces->right || !faces->area ||
+      !faces->nx || !faces->ny || !faces->nz || !faces->fx || !faces->fy || !faces->fz)
+    return fail(ctx, RT_INVALID_ARG, "mesh array is NULL");
+  free_all(ctx);
+  const rt_status st = build_mesh(ctx, cells, faces);
+  if (st) free_all(ctx);   // a refused mesh holds no memory
+  return st;
 }
 
 rt_status rt_set_gas(rt_ctx* ctx, const double* nH, const double* x5, const double* T) {
