@@ -84,7 +84,8 @@ __device__ __forceinline__ double rint_away(double x) { return round(x); }
 __device__ __forceinline__ float rint_away(float x) { return roundf(x); }
 
 // Periodic box of side L (0: not periodic) with the high words of 0.4999 L,
-// 0.5001 L and 1.4999 L.
+// 0.5001 L and 1.4999 L (an infinite L has none: the expression below, NaN, which
+// the least-squares matrix's check refuses).
 struct Box {
   double L;
   int h_in, h_out, h_two;
@@ -95,6 +96,7 @@ inline Box make_box(double L) {
     std::memcpy(&b, &v, sizeof b);
     return (int)(b >> 32);
   };
+  if (L > 0x1.fffffffffffffp1023) return Box{L, 0, 0x7FFFFFFF, 0};
   return Box{L, hi(0.4999 * L), hi(0.5001 * L), hi(1.4999 * L)};
 }
 
