@@ -282,7 +282,9 @@ const char *rt_fp64_peak_last_error(void);
  * memory); anything else, device memory of another GPU included, gets
  * RT_INVALID_ARG before anything is enqueued.  The arrays must describe a
  * valid mesh (ids in range); they are not checked.
- * At most 262144 cells; larger meshes get RT_INVALID_ARG.  Nothing is
+ * At most 262144 cells; larger meshes get RT_INVALID_ARG and belong in a
+ * context.  Fastest with lengths between 1e-18 and 1e18 (a third more time
+ * with the limiter on beyond; the results do not depend on it).  Nothing is
  * allocated and no device memory outside the caller's arrays is used, so
  * calls with different outputs may overlap.  Asynchronous on stream;
  * host-side errors and failed launches of its own kernels are returned as

@@ -127,7 +127,7 @@ __global__ void __launch_bounds__(256) k_adj_face(AdjArgs a) {
 }
 
 // The gradients before the limiter, its factors and the limiting faces come
-// from k_grad's record of the same state (192 bytes read instead of the
+// from k_grad's record of the same state (160 bytes read instead of the
 // least-squares sums and a quotient per face and component formed again, which
 // were two thirds of this kernel's FP64 instructions).
 __global__ void __launch_bounds__(256) k_adj_cellgrad(AdjArgs a) {

@@ -128,8 +128,8 @@ struct RatesF {
 // Precision conversions of the mixed chemistry.  IntCvt: assembled on the
 // integer pipe (d2f_int, f2d_int), for the first pass over every cell, where
 // the FP64 pipe bounds the kernel; otherwise the hardware's conversions, for
-// the worklist pass, where a few stiff cells run long serial chains of
-// attempts and an attempt's latency counts: one instruction instead of ten.
+// the worklist pass by threads, where a few stiff cells run long serial chains
+// of attempts and an attempt's latency counts: one instruction instead of ten.
 // The two round alike (to nearest) but for exact ties and subnormal values.
 template <bool IntCvt> __device__ __forceinline__ float to_f(double x) {
   if constexpr (IntCvt) return d2f_int(x);
@@ -375,7 +375,7 @@ struct GasState {
 
 // IntCvt (the first attempt, over the common length): c dt sigma comes with
 // the kernel's arguments instead of being multiplied out in the optical
-// depths, the photoionisation rates and the photon removal: 96 FP64
+// depths, the photoionisation rates and the photon removal: 92 FP64
 // instructions per attempt instead of 109, of which the first pass is made.
 template <bool IntCvt>
 __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double dt, const GasState& s,

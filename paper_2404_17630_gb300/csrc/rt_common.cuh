@@ -80,9 +80,6 @@ template <> __device__ __forceinline__ d4 ld4<double>(const d4* p) { return *p; 
 
 template <class R> __device__ __forceinline__ R mk(double v) { return static_cast<R>(v); }
 
-__device__ __forceinline__ double rint_away(double x) { return round(x); }
-__device__ __forceinline__ float rint_away(float x) { return roundf(x); }
-
 // Periodic box of side L (0: not periodic) with the high words of 0.4999 L,
 // 0.5001 L and 1.4999 L (an infinite L has none: the expression below, NaN, which
 // the least-squares matrix's check refuses).

@@ -1412,10 +1412,11 @@ __global__ void k_reciprocal(int n, const double* __restrict__ in, double* out) 
 // -- and finishes the cells it accepts; the cells it rejects go to a
 // worklist that k_chem_rest works through with the adaptive loop.  Each
 // cell makes the attempts one pass would make: the first pass converts
-// between FP32 and FP64 on the integer pipe (it is bound by the FP64 pipe),
-// the worklist pass with the hardware's conversions (a few stiff cells run
-// long serial chains of attempts there, bound by an attempt's latency); the
-// two round alike but for exact ties and subnormal values.  The attempts
+// between FP32 and FP64 on the integer pipe (it is bound by the FP64 pipe), as
+// do the worklist's groups of lanes, its threads with the hardware's
+// conversions (a few stiff cells run long serial chains of attempts there,
+// bound by an attempt's latency); the two round alike but for exact ties and
+// subnormal values.  The attempts
 // carry N and the gas only; the flux is read at the end and scaled by the
 // product of the accepted photon factors.
 

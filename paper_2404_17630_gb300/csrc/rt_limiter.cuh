@@ -72,11 +72,11 @@ __device__ __forceinline__ bool scaled_f32(const double g[3], float o[3]) {
 // the matrix folded into the weights: 0.85 -> 0.52 ms per launch at 250,047
 // cells, 142 -> 82 us at 262,144 cells of six faces and one bin).  A leader
 // beyond the test's bound for the largest |x_f|, by the same margin, also passes
-// its own test, and nothing more is to be tested: rounding is monotone.  Where a lead is smaller
-// (faces that tie by symmetry; a leader within the band of zero) every face's
-// product is formed in FP64 and, where an extreme does not clear the bound,
-// tested.  A component without gradient has no extremes.  at[2q], at[2q + 1]: the
-// first face that attains dpos[q], dneg[q].
+// its own test, and nothing more is to be tested: rounding is monotone.  Where a
+// lead is smaller (faces that tie by symmetry; a leader within the band of zero)
+// every face's product is formed in FP64 and, where an extreme does not clear the
+// bound, tested.  A component without gradient has no extremes.  at[2q],
+// at[2q + 1]: the first face that attains dpos[q], dneg[q].
 __device__ __forceinline__ void lim_extremes(const d4* __restrict__ xs, const float4* __restrict__ xf, int k0, int k1,
                                              const double gr[4][3], double eps2, double X, float xm,
                                              double dpos[4], double dneg[4], int at[8]) {

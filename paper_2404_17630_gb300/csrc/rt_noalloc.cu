@@ -18,8 +18,8 @@
 
 namespace {
 
+// The interface's limit on the mesh (what the entry point has always refused).
 constexpr int64_t kNoallocMaxCells = 262144;
-constexpr int kMaxDevices = 64;
 
 // Kernel launch that returns this launch's own status (a triple-chevron
 // launch only leaves it in the thread's last-error slot, where an error the
@@ -263,10 +263,10 @@ rt_status rt_gradients_noalloc(const rt_cells* cells, const rt_faces* faces, con
   const int64_t C = cells->n, F = faces->n;
   if (C <= 0 || F <= 0) return set_err(RT_INVALID_ARG, "rt_gradients_noalloc: empty mesh");
   if (C > kNoallocMaxCells)
-    return set_err(RT_INVALID_ARG, "rt_gradients_noalloc: more than 262144 cells (size of its static scratch)");
+    return set_err(RT_INVALID_ARG, "rt_gradients_noalloc: more than 262144 cells (larger meshes through a context)");
   if (F > (1LL << 29)) return set_err(RT_INVALID_ARG, "rt_gradients_noalloc: too many faces");
   int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
+  if (cudaGetDevice(&dev) != cudaSuccess) {
     cudaGetLastError();
     return set_err(RT_CUDA, "rt_gradients_noalloc: no current device");
   }
