@@ -450,6 +450,157 @@ rt_status need_mesh(rt_ctx* ctx) {
   return RT_OK;
 }
 
+// ---- active sets -----------------------------------------------------------
+
+// Small meshes keep their active masks on the host as well and compare them
+// there, and the smallest build the lists there: a launch, a copy and a wait
+// apiece cost more than the work.  us per call, host / device: a known mask
+// 12 / 31 at 1,000 cells, 13 / 33 at 8,000, above that the copy of a device mask
+// and the comparison grow; a new one 47 / 153 at 216 cells, 76 / 161 at 1,000 and,
+// with an allocation and a copy per list, 415 / 162 at 8,000.
+constexpr int kMaskOnHost = 8192, kListsOnHost = 2048;
+
+// A new mask into mask_norm (0 / 1, padded with ones to whole words) and against
+// the kept ones; on the legacy stream, as the copy, so that a device mask is read
+// after the work that wrote it.
+rt_status match_mask(rt_ctx* ctx, const uint8_t* active, unsigned* differs) {
+  static_assert(KnownMasks::kMax == rt_ctx::kMaxActSets, "one bit per kept set");
+  const int C = ctx->C;
+  const size_t padded = ((size_t)C + 15) / 16 * 16;
+  KnownMasks known{};
+  for (int j = 0; j < rt_ctx::kMaxActSets; ++j) known.m[j] = ctx->sets[j].valid ? ctx->sets[j].mask : nullptr;
+  CK(cudaMemcpy(ctx->mask_in, active, (size_t)C, is_device_ptr(active) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice),
+     "active mask");
+  CK(cudaMemsetAsync(ctx->mask_res, 0, sizeof(unsigned), cudaStreamLegacy), "active mask");
+  k_match_mask<<<nblk((long long)padded / 16), kThreads, 0, cudaStreamLegacy>>>(C, ctx->mask_in, ctx->mask_norm, known,
+                                                                                 ctx->mask_res);
+  rt_status st = launched(ctx, "active mask");
+  if (st) return st;
+  CK(cudaMemcpy(differs, ctx->mask_res, sizeof(unsigned), cudaMemcpyDeviceToHost), "active mask");
+  return RT_OK;
+}
+
+// The lists of the mask in mask_norm, built on the device.
+rt_status device_lists(rt_ctx* ctx, rt_ctx::ActSet& a) {
+  rt_status st;
+  const int C = ctx->C, F = ctx->F;
+  const size_t padded = ((size_t)C + 15) / 16 * 16;
+  // flags and counts first, the lists once their lengths are known.  The
+  // flags of faces and blocks and the partial counts lie in the staging
+  // buffer (7 F doubles at least).
+  const int nblock = (C + kGradCells - 1) / kGradCells;
+  auto parts = [](int n) { return (n + kScan - 1) / kScan; };
+  uint8_t* face = (uint8_t*)ctx->stage;
+  uint8_t* block = face + ((size_t)F + 15) / 16 * 16;
+  int32_t* sums = (int32_t*)(block + ((size_t)nblock + 15) / 16 * 16);
+  int32_t *s_act = sums, *s_touched = s_act + parts(C) + 1, *s_face = s_touched + parts(C) + 1,
+          *s_block = s_face + parts(F) + 1;
+  int* cap = (int*)ctx->mask_res;
+  cudaStream_t q = cudaStreamLegacy;
+  uint8_t* touched = ctx->mask_in;   // its contents are in mask_norm
+  CK(cudaMemsetAsync(touched, 0, (size_t)C, q), "active lists");
+  CK(cudaMemsetAsync(cap, 0, sizeof(int), q), "active lists");
+  k_set_faces<<<nblk(F), kThreads, 0, q>>>(F, ctx->lr, ctx->mask_norm, face, touched);
+  k_set_blocks<<<nblk(nblock), kThreads, 0, q>>>(nblock, C, kGradCells, touched, block);
+  struct { int n; const uint8_t* flag; int32_t* sums; } job[] = {
+      {C, ctx->mask_norm, s_act}, {C, touched, s_touched}, {F, face, s_face}, {nblock, block, s_block}};
+  for (auto& j : job) {
+    k_flag_count<<<parts(j.n), kScan, 0, q>>>(j.n, j.flag, j.sums);
+    k_scan_sums<<<1, kScan, 0, q>>>(parts(j.n), j.sums);
+  }
+  if ((st = launched(ctx, "active lists"))) return st;
+  int count[4] = {};
+  for (int i = 0; i < 4; ++i)
+    CK(cudaMemcpyAsync(count + i, job[i].sums + parts(job[i].n), sizeof(int), cudaMemcpyDeviceToHost, q), "active lists");
+  CK(cudaStreamSynchronize(q), "active lists");
+  Arena ar;
+  ar.add(&a.act_cells, count[0]); ar.add(&a.touched_cells, count[1]); ar.add(&a.act_faces, count[2]);
+  ar.add(&a.grad_blocks, count[3]); ar.add(&a.touched, C); ar.add(&a.mask, padded);
+  void* p = nullptr;
+  cudaError_t e = cudaMalloc(&p, ar.bytes);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "active lists");
+  a.allocs.push_back(p);
+  ar.place(p);
+  int32_t* list[] = {a.act_cells, a.touched_cells, a.act_faces, a.grad_blocks};
+  for (int i = 0; i < 4; ++i)
+    k_flag_list<<<parts(job[i].n), kScan, 0, q>>>(job[i].n, job[i].flag, job[i].sums, list[i]);
+  // staged gradients over the touched list: the face records of the
+  // largest block of kGradCells list entries must fit in shared memory
+  if (mixed(ctx) && ctx->grad_cap > 0 && count[1] > 0)
+    k_list_cap<<<nblk((count[1] + kGradCells - 1) / kGradCells), kThreads, 0, q>>>(count[1], kGradCells,
+                                                                                   a.touched_cells, ctx->off, cap);
+  int cap_list = 0;
+  if ((st = launched(ctx, "active lists"))) return st;
+  CK(cudaMemcpyAsync(a.touched, touched, (size_t)C, cudaMemcpyDeviceToDevice, q), "active lists");
+  CK(cudaMemcpyAsync(a.mask, ctx->mask_norm, padded, cudaMemcpyDeviceToDevice, q), "active lists");
+  CK(cudaMemcpyAsync(&cap_list, cap, sizeof(int), cudaMemcpyDeviceToHost, q), "active lists");
+  CK(cudaStreamSynchronize(q), "active lists");
+  if (2 * (size_t)cap_list * sizeof(float4) > kGradSmemMax) cap_list = 0;
+  a.n_act = count[0];
+  a.n_touched = count[1];
+  a.n_act_faces = count[2];
+  a.n_grad_blocks = count[3];
+  a.grad_cap_list = cap_list;
+  return RT_OK;
+}
+
+// The lists of the mask m, built on the host.
+rt_status host_lists(rt_ctx* ctx, const std::vector<uint8_t>& m, rt_ctx::ActSet& a) {
+  const int C = ctx->C, F = ctx->F;
+  std::vector<int2> lr(F);
+  CK(cudaMemcpy(lr.data(), ctx->lr, (size_t)F * sizeof(int2), cudaMemcpyDeviceToHost), "active lists");
+  std::vector<int32_t> act, touched, face, block, deg(C, 0);
+  std::vector<uint8_t> flag(C, 0);
+  for (int i = 0; i < C; ++i)
+    if (m[i]) act.push_back(i);
+  for (int f = 0; f < F; ++f) {
+    const int2 c = lr[f];
+    deg[c.x]++;
+    deg[c.y]++;
+    if (m[c.x] || m[c.y]) {
+      face.push_back(f);
+      flag[c.x] = flag[c.y] = 1;
+    }
+  }
+  for (int i = 0; i < C; ++i)
+    if (flag[i]) {
+      touched.push_back(i);
+      if (block.empty() || block.back() != i / kGradCells) block.push_back(i / kGradCells);
+    }
+  // one buffer, filled here and copied at once
+  Arena ar;
+  ar.add(&a.act_cells, act.size()); ar.add(&a.touched_cells, touched.size()); ar.add(&a.act_faces, face.size());
+  ar.add(&a.grad_blocks, block.size()); ar.add(&a.touched, C);
+  std::vector<uint8_t> all(ar.bytes);
+  const std::pair<const void*, size_t> part[] = {{act.data(), 4 * act.size()}, {touched.data(), 4 * touched.size()},
+                                                 {face.data(), 4 * face.size()}, {block.data(), 4 * block.size()},
+                                                 {flag.data(), (size_t)C}};
+  for (size_t q = 0; q < ar.at.size(); ++q)
+    if (part[q].second) std::memcpy(all.data() + ar.at[q].second, part[q].first, part[q].second);
+  void* p = nullptr;
+  CK(cudaMalloc(&p, ar.bytes), "active lists");
+  a.allocs.push_back(p);
+  ar.place(p);
+  CK(cudaMemcpy(p, all.data(), ar.bytes, cudaMemcpyHostToDevice), "active lists");
+  // a copy from pageable memory may still be on its way when the call returns,
+  // and the context's stream need not wait for the legacy one
+  CK(cudaStreamSynchronize(cudaStreamLegacy), "active lists");
+  int cap = 0;
+  if (mixed(ctx) && ctx->grad_cap > 0)
+    for (size_t j0 = 0; j0 < touched.size(); j0 += kGradCells) {
+      int sum = 0;
+      for (size_t j = j0; j < std::min(j0 + kGradCells, touched.size()); ++j) sum += deg[touched[j]];
+      cap = std::max(cap, sum);
+    }
+  if (2 * (size_t)cap * sizeof(float4) > kGradSmemMax) cap = 0;
+  a.n_act = (int)act.size();
+  a.n_touched = (int)touched.size();
+  a.n_act_faces = (int)face.size();
+  a.n_grad_blocks = (int)block.size();
+  a.grad_cap_list = cap;
+  return RT_OK;
+}
+
 // rt_init_mesh after the checks of its arguments, on a context without a mesh.
 rt_status build_mesh(rt_ctx* ctx, const rt_cells* cells, const rt_faces* faces) {
   const int C = (int)cells->n, F = (int)faces->n, B = ctx->B;
@@ -776,28 +927,28 @@ rt_status rt_set_active(rt_ctx* ctx, const uint8_t* active) {
     use_set(ctx, -1);
     return RT_OK;
   }
-  // compared on the device with the masks seen recently, which keep their
-  // lists and step graphs; on the legacy stream, as the copy, so that a device
-  // mask is read after the work that wrote it
-  static_assert(KnownMasks::kMax == rt_ctx::kMaxActSets, "one bit per kept set");
-  const size_t padded = ((size_t)C + 15) / 16 * 16;
-  KnownMasks known{};
-  for (int j = 0; j < rt_ctx::kMaxActSets; ++j) known.m[j] = ctx->sets[j].valid ? ctx->sets[j].mask : nullptr;
-  unsigned res = 0;
-  CK(cudaMemcpy(ctx->mask_in, active, (size_t)C, is_device_ptr(active) ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice),
-     "active mask");
-  CK(cudaMemsetAsync(ctx->mask_res, 0, sizeof(unsigned), cudaStreamLegacy), "active mask");
-  k_match_mask<<<nblk((long long)padded / 16), kThreads, 0, cudaStreamLegacy>>>(C, ctx->mask_in, ctx->mask_norm, known,
-                                                                                 ctx->mask_res);
-  if ((st = launched(ctx, "active mask"))) return st;
-  CK(cudaMemcpy(&res, ctx->mask_res, sizeof(unsigned), cudaMemcpyDeviceToHost), "active mask");
-  if (!(res >> rt_ctx::kMaxActSets & 1u)) {
+  // compared with the masks seen recently, which keep their lists and step
+  // graphs
+  std::vector<uint8_t> m;
+  unsigned differs = 0;   // bit j: from the mask of set j; bit kMaxActSets: from all ones
+  if (C <= kMaskOnHost) {
+    m.resize(C);
+    if (is_device_ptr(active)) CK(cudaMemcpy(m.data(), active, (size_t)C, cudaMemcpyDeviceToHost), "active mask");
+    else std::memcpy(m.data(), active, (size_t)C);
+    for (uint8_t& v : m) v = v != 0;
+    if (std::memchr(m.data(), 0, (size_t)C)) differs |= 1u << rt_ctx::kMaxActSets;
+    for (int j = 0; j < rt_ctx::kMaxActSets; ++j)
+      if (ctx->sets[j].valid && ctx->sets[j].host != m) differs |= 1u << j;
+  } else if ((st = match_mask(ctx, active, &differs))) {
+    return st;
+  }
+  if (!(differs >> rt_ctx::kMaxActSets & 1u)) {
     use_set(ctx, -1);
     return RT_OK;
   }
   int k = -1;
   for (int j = 0; j < rt_ctx::kMaxActSets && k < 0; ++j)
-    if (ctx->sets[j].valid && !(res >> j & 1u)) k = j;
+    if (ctx->sets[j].valid && !(differs >> j & 1u)) k = j;
   if (k < 0) {
     // a free slot, else the least recently used one
     for (int j = 0; j < rt_ctx::kMaxActSets && k < 0; ++j)
@@ -809,70 +960,24 @@ rt_status rt_set_active(rt_ctx* ctx, const uint8_t* active) {
     }
     rt_ctx::ActSet& a = ctx->sets[k];
     free_set(a);
-    // flags and counts first, the lists once their lengths are known.  The
-    // flags of faces and blocks and the partial counts lie in the staging
-    // buffer (7 F doubles at least).
-    const int nblock = (C + kGradCells - 1) / kGradCells;
-    auto parts = [](int n) { return (n + kScan - 1) / kScan; };
-    uint8_t* face = (uint8_t*)ctx->stage;
-    uint8_t* block = face + ((size_t)F + 15) / 16 * 16;
-    int32_t* sums = (int32_t*)(block + ((size_t)nblock + 15) / 16 * 16);
-    int32_t *s_act = sums, *s_touched = s_act + parts(C) + 1, *s_face = s_touched + parts(C) + 1,
-            *s_block = s_face + parts(F) + 1;
-    int* cap = (int*)ctx->mask_res;
-    cudaStream_t q = cudaStreamLegacy;
-    uint8_t* touched = ctx->mask_in;   // its contents are in mask_norm
-    CK(cudaMemsetAsync(touched, 0, (size_t)C, q), "active lists");
-    CK(cudaMemsetAsync(cap, 0, sizeof(int), q), "active lists");
-    k_set_faces<<<nblk(F), kThreads, 0, q>>>(F, ctx->lr, ctx->mask_norm, face, touched);
-    k_set_blocks<<<nblk(nblock), kThreads, 0, q>>>(nblock, C, kGradCells, touched, block);
-    struct { int n; const uint8_t* flag; int32_t* sums; } job[] = {
-        {C, ctx->mask_norm, s_act}, {C, touched, s_touched}, {F, face, s_face}, {nblock, block, s_block}};
-    for (auto& j : job) {
-      k_flag_count<<<parts(j.n), kScan, 0, q>>>(j.n, j.flag, j.sums);
-      k_scan_sums<<<1, kScan, 0, q>>>(parts(j.n), j.sums);
+    if (C <= kListsOnHost) {
+      st = host_lists(ctx, m, a);
+    } else {
+      if (!m.empty()) {
+        // as match_mask leaves it: padded with ones to whole words
+        std::vector<uint8_t> padded(m);
+        padded.resize(((size_t)C + 15) / 16 * 16, 1);
+        cudaError_t e = cudaMemcpy(ctx->mask_norm, padded.data(), padded.size(), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) st = cuda_fail(ctx, e, "active mask");
+      }
+      if (!st) st = device_lists(ctx, a);
     }
-    if ((st = launched(ctx, "active lists"))) return st;
-    int count[4] = {};
-    for (int i = 0; i < 4; ++i)
-      CK(cudaMemcpyAsync(count + i, job[i].sums + parts(job[i].n), sizeof(int), cudaMemcpyDeviceToHost, q), "active lists");
-    CK(cudaStreamSynchronize(q), "active lists");
-    Arena ar;
-    ar.add(&a.act_cells, count[0]); ar.add(&a.touched_cells, count[1]); ar.add(&a.act_faces, count[2]);
-    ar.add(&a.grad_blocks, count[3]); ar.add(&a.touched, C); ar.add(&a.mask, padded);
-    void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, ar.bytes);
-    if (e != cudaSuccess) {
-      free_set(a);
-      use_set(ctx, -1);
-      return cuda_fail(ctx, e, "active lists");
-    }
-    a.allocs.push_back(p);
-    ar.place(p);
-    int32_t* list[] = {a.act_cells, a.touched_cells, a.act_faces, a.grad_blocks};
-    for (int i = 0; i < 4; ++i)
-      k_flag_list<<<parts(job[i].n), kScan, 0, q>>>(job[i].n, job[i].flag, job[i].sums, list[i]);
-    // staged gradients over the touched list: the face records of the
-    // largest block of kGradCells list entries must fit in shared memory
-    if (mixed(ctx) && ctx->grad_cap > 0 && count[1] > 0)
-      k_list_cap<<<nblk((count[1] + kGradCells - 1) / kGradCells), kThreads, 0, q>>>(count[1], kGradCells,
-                                                                                     a.touched_cells, ctx->off, cap);
-    int cap_list = 0;
-    if ((st = launched(ctx, "active lists"))) {
+    if (st) {
       free_set(a);
       use_set(ctx, -1);
       return st;
     }
-    CK(cudaMemcpyAsync(a.touched, touched, (size_t)C, cudaMemcpyDeviceToDevice, q), "active lists");
-    CK(cudaMemcpyAsync(a.mask, ctx->mask_norm, padded, cudaMemcpyDeviceToDevice, q), "active lists");
-    CK(cudaMemcpyAsync(&cap_list, cap, sizeof(int), cudaMemcpyDeviceToHost, q), "active lists");
-    CK(cudaStreamSynchronize(q), "active lists");
-    if (2 * (size_t)cap_list * sizeof(float4) > kGradSmemMax) cap_list = 0;
-    a.n_act = count[0];
-    a.n_touched = count[1];
-    a.n_act_faces = count[2];
-    a.n_grad_blocks = count[3];
-    a.grad_cap_list = cap_list;
+    a.host.swap(m);
     a.valid = true;
   }
   use_set(ctx, k);

@@ -85,6 +85,7 @@ struct rt_ctx {
     bool valid = false;
     uint64_t used = 0;
     uint8_t* mask = nullptr;   // device: 0 / 1 per cell, padded with ones to 16
+    std::vector<uint8_t> host; // the same on the host (small meshes)
     int32_t *act_cells = nullptr, *touched_cells = nullptr, *act_faces = nullptr, *grad_blocks = nullptr;
     uint8_t* touched = nullptr;
     int n_act = 0, n_touched = 0, n_act_faces = 0, n_grad_blocks = 0;
