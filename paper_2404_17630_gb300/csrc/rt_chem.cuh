@@ -231,10 +231,11 @@ __device__ __forceinline__ double largest_change(const double a[n], const double
   return f;
 }
 
-// x, and 0 where it is negative (NaN stays), on the integer pipe.
+// x, and 0 where it is negative (NaN stays), on the integer pipe (from the high
+// word: a test on all the bits is compiled into an FP64 comparison).
 __device__ __forceinline__ double clamp_neg(double x) {
-  const long long b = __double_as_longlong(x);
-  return b < 0 && (b & 0x7FFFFFFFFFFFFFFFLL) <= 0x7FF0000000000000LL ? 0.0 : x;
+  const unsigned h = (unsigned)__double2hiint(x) ^ 0x80000000u;   // of -x
+  return h <= 0x7FF00000u ? 0.0 : x;
 }
 
 // |x| on the integer pipe.
