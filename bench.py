@@ -401,7 +401,7 @@ FP64_FLOP = {
 # rate against the stream's (peak FLOP / 2 per DFMA) is the pipe's use.
 FP64_INST = {
     "mixed": {"k_chem": (92.1, "attempt")},
-    "fp64": {"k_chem": (553.2, "attempt"), "k_grad": (1106.0, "cell"), "k_flux": (2213.0, "cell"),
+    "fp64": {"k_chem": (553.2, "attempt"), "k_grad": (1103.0, "cell"), "k_flux": (2213.0, "cell"),
              "k_gather": (282.4, "cell")},
 }
 # Fallback FP64 peak from unit counts and clock, used only when the
