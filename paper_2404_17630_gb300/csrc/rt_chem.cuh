@@ -243,6 +243,14 @@ __device__ __forceinline__ double no_sign(double x) {
   return __hiloint2double(__double2hiint(x) & 0x7FFFFFFF, __double2loint(x));
 }
 
+// x <= 0 (not NaN), on the integer pipe.  A bin that enters the attempts of the
+// mixed path so leaves the first accepted one with N = 0 and without flux, and
+// stays there; the others never come to N < 0.
+__device__ __forceinline__ bool unlit(double x) {
+  const unsigned h = (unsigned)__double2hiint(x);
+  return (h ^ 0x80000000u) <= 0x7FF00000u || (h | (unsigned)__double2loint(x)) == 0u;
+}
+
 // One semi-implicit photochemistry attempt over dt from s into t; returns the
 // largest relative change f of the substep rule.  Steps: radiation level
 // over the step (implicit in N, absorbers at the start); photoionisation
@@ -455,10 +463,11 @@ __device__ float photochem_attempt_mixed(const ChemParams& P, double nH, double 
       const double taup = IntCvt ? suma : cdt * suma;
       // N' = max(N - removed, 0) and no flux where N <= 0, as in the FP64
       // attempt: the factor is clamped on the integer pipe (a double's bits
-      // order like the value where it is positive), and a zero keeps no sign
+      // order like the value where it is positive), and a zero keeps no sign.
+      // In the loop over attempts N <= 0 is the caller's (unlit).
       double sc = fma(-taup, inv1pt[b], 1.0);
-      sc = __double_as_longlong(sc) > 0 && __double_as_longlong(s.N[b]) > 0 ? sc : 0.0;
-      t.N[b] = no_sign(s.N[b] * sc);
+      sc = __double_as_longlong(sc) > 0 && (!IntCvt || __double_as_longlong(s.N[b]) > 0) ? sc : 0.0;
+      t.N[b] = IntCvt ? no_sign(s.N[b] * sc) : s.N[b] * sc;
       if (heat) {
         float ea = 0.0f;
 #pragma unroll
@@ -524,7 +533,10 @@ template <bool IntCvt>
 __device__ int chemistry_mixed(const ChemParams& P, double nH, double dt_sub, GasState& s,
                                float S[kMaxBins], bool* capped, double dt0, int n0) {
   double rem = dt_sub, dt = dt0;
-  int n = n0, acc = 0;
+  int n = n0, acc = 0, dark = 0;
+#pragma unroll
+  for (int b = 0; b < kMaxBins; ++b)
+    if (b < P.B && unlit(s.N[b])) dark |= 1 << b;
   GasState t;
   float sc[kMaxBins];
   *capped = false;
@@ -540,6 +552,11 @@ __device__ int chemistry_mixed(const ChemParams& P, double nH, double dt_sub, Ga
     s = t;
 #pragma unroll
     for (int b = 0; b < kMaxBins; ++b) S[b] = acc ? S[b] * sc[b] : sc[b];
+    if (dark) {
+#pragma unroll
+      for (int b = 0; b < kMaxBins; ++b)
+        if (dark >> b & 1) { s.N[b] = 0.0; S[b] = 0.0f; }
+    }
     ++acc;
     rem = (__double_as_longlong(dt) == __double_as_longlong(rem)) ? 0.0 : rem - dt;
     const float grow = f > 0.0f ? fminf(__fdividef(fs, f), 2.0f) : 2.0f;

@@ -250,10 +250,13 @@ __device__ __forceinline__ auto group_attempt(const ChemParams& P, const Fit& fi
   // photons of the lane's bin: removed as the ionisations were credited
   const double suma = fma(g.sd[2], t.x[3], fma(g.sd[1], t.x[2], g.sd[0] * t.x[0]));
   double sc = fma(-(cdt * suma), inv1pt, 1.0);
-  const bool lit = positive(sc) && positive(s.N);
-  if constexpr (!Mixed) t.N = clamp_neg(s.N * sc);
-  sc = lit ? sc : 0.0;
-  if constexpr (Mixed) t.N = no_sign(s.N * sc);
+  if constexpr (Mixed) {
+    sc = positive(sc) ? sc : 0.0;   // N <= 0 is the caller's (unlit)
+    t.N = s.N * sc;
+  } else {
+    t.N = clamp_neg(s.N * sc);
+    sc = positive(sc) && positive(s.N) ? sc : 0.0;
+  }
   t.T = s.T;
   V f = V(0);
   // change of the lane's abundance (lanes 0-4)

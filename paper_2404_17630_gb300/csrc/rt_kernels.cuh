@@ -1584,6 +1584,7 @@ __device__ __forceinline__ void rest_groups(const CellArgs& a, const ChemParams&
   group_cell(P, l, 1.0, g);
   double rem = 0.0, dt = 0.0;
   float S = 1.0f;
+  bool dark = false;   // the lane's bin came with N <= 0
   int i = 0, n = 0;
   const float fmx = (float)P.f_max, fs = (float)P.f_s;
   auto load = [&](int k) {
@@ -1593,12 +1594,14 @@ __device__ __forceinline__ void rest_groups(const CellArgs& a, const ChemParams&
     for (int q = 0; q < 5; ++q) s.x[q] = a.x5[q * C + i];
     s.T = a.T[i];
     s.N = l < B ? a.radN[(size_t)i * B + l] : 0.0;
+    dark = unlit(s.N);
     rem = a.dt;
     dt = a.dt * f2d_int(__fdividef(fs, w.f1[k]));
-    S = 1.0f;
+    S = dark ? 0.0f : 1.0f;
     n = 1;
   };
   auto store = [&]() {
+    if (__double_as_longlong(rem) == __double_as_longlong(a.dt)) S = 1.0f;   // nothing was accepted
     if (l < B) {
       const size_t r = (size_t)i * B + l;
       a.radN[r] = s.N;
@@ -1637,6 +1640,7 @@ __device__ __forceinline__ void rest_groups(const CellArgs& a, const ChemParams&
           dt = dt * (double)__fdividef(fs, f);
         } else {
           s = t;
+          s.N = dark ? 0.0 : t.N;
           S *= d2f_int(sc);
           rem = __double_as_longlong(dt) == __double_as_longlong(rem) ? 0.0 : rem - dt;
           dt = dt * (double)(f > 0.0f ? fminf(__fdividef(fs, f), 2.0f) : 2.0f);

@@ -133,3 +133,24 @@ def test_beam_mixed():
     rt.sync()
     e = _errors(rt, o, cfg)
     assert max(e.values()) < 1e-4, e
+
+
+@pytest.mark.parametrize("prec,tol", [("fp64", 1e-12), ("mixed", 1e-4)])
+@pytest.mark.parametrize("most", [1, 2])
+def test_cap(prec, tol, most):
+    """Cells that reach the cap on attempts, some before one is accepted: those keep N < 0 and their flux."""
+    from paper_2404_17630_gb300.rt import RTError
+    mesh, cfg, st = _negative(6)
+    cfg = dict(cfg, max_substeps=most)
+    o, rt = make_oracle(mesh, cfg, st), _gpu(mesh, cfg, st, precision=prec, gather_sum=1)
+    dt = 0.9 * o.max_dt()
+    assert o.thermochemistry(dt) == 4
+    rt.thermochemistry(dt)
+    with pytest.raises(RTError, match="max_substeps"):
+        rt.sync()
+    g = rt.fields()
+    N, fr = o.radiation()
+    x5, T = o.gas()
+    assert N.min() < 0
+    for a, b in ((g["N"], N), (g["F"] / cfg["c_red"], fr), (g["x5"], x5), (g["T"], T)):
+        assert np.abs(a - b).max() < tol * np.abs(b).max()
